@@ -92,7 +92,8 @@ typedef struct {
     double chi2_match_max;     /* chi2_match < 2 */
     int32_t velo_unique;       /* 1: a VELO segment keeps only its best seed */
     /* launch tuning (no effect on results) */
-    int32_t threads_seed;      /* threads per CTA of the seeding kernel: 64, 128, 256, 512 */
+    int32_t threads_seed;      /* threads per CTA of the seeding kernel: 64, 128, 256, 512 (batches that
+                                * leave SMs idle take larger CTAs unless ctas_per_sm is set) */
     int32_t threads_build;     /* threads per CTA of the container kernel */
     int32_t threads_match;     /* threads per CTA of the matching kernel */
     int32_t ctas_per_sm;       /* persistent CTAs per SM (0 = occupancy maximum) */
@@ -310,9 +311,8 @@ int st_set_ghost_nn(st_ctx* ctx, const float* weights, int32_t n);
  * CUDA graph (persistent, work-queue kernels).  Scratch must be reserved
  * first (st_reserve).  The arguments' pointers must stay valid while the
  * graph exists.  *out receives the graph; launch with st_graph_launch.
- * With threads_seed <= 256, iter_mode 0 and no final selection the matching
- * runs inside the seeding kernel (each event as soon as its two halves are
- * seeded); the outputs are those of the two calls.  If that kernel ever gave
+ * With iter_mode 0 and no final selection the matching runs inside the
+ * seeding kernel (each event as soon as its two halves are seeded); the outputs are those of the two calls.  If that kernel ever gave
  * up a (bounded) wait for an event being seeded, which a correct run cannot
  * do, every event of the launch gets status ST_TIMEOUT.  The serving pipeline
  * runs batches the same way. */

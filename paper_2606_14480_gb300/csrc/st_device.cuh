@@ -17,6 +17,7 @@ constexpr int kSlotsPerHalf = 12;  // 6 x-layer zones, then 6 stereo zones
 constexpr int kZoffStride = 25;    // per event: 24 slot starts + end
 constexpr int kMasks = 7;          // x-layer hit patterns with >= 5 hits
 constexpr int kMaxThreads = 512;
+constexpr int kScanInts = 64;  // shared ints of a one-barrier block scan: two halves of a partial sum per warp
 
 // Container order of an event: half-major; within a half the x-layers
 // (0,3,4,7,8,11) then the stereo layers (1,2,5,6,9,10), each sorted by x.
@@ -52,7 +53,6 @@ struct DevParams {
     float G[kMasks][3][6]; // least-squares gain per x-hit pattern
     int mask_index[64];    // 6-bit x-hit pattern -> G index, -1 if < 5 hits
     int uv_init[2];        // stereo slot of the initial layer of each pass
-    int uv_rem[2][5];      // the other stereo slots of each pass, ascending z
     int n_uv_min;
     float uv_tol;
     float uv_ylo[2], uv_yhi[2];  // first-layer y window per half
@@ -100,56 +100,6 @@ __device__ __forceinline__ void two_prod(float a, float b, float& p, float& e) {
 }
 
 // ---------------------------------------------------------------------------
-// searches over an ascending float array
-// ---------------------------------------------------------------------------
-
-// first index i in [0, n) with a[i] >= v (n if none)
-__device__ __forceinline__ int lower_bound_f(const float* a, int n, float v) {
-    int lo = 0, len = n;
-    while (len > 0) {
-        int h = len >> 1;
-        if (a[lo + h] < v) {
-            lo += h + 1;
-            len -= h + 1;
-        } else {
-            len = h;
-        }
-    }
-    return lo;
-}
-
-// first index i in [0, n) with a[i] > v (n if none)
-__device__ __forceinline__ int upper_bound_f(const float* a, int n, float v) {
-    int lo = 0, len = n;
-    while (len > 0) {
-        int h = len >> 1;
-        if (!(v < a[lo + h])) {
-            lo += h + 1;
-            len -= h + 1;
-        } else {
-            len = h;
-        }
-    }
-    return lo;
-}
-
-// largest t in [0, n) with s[t] <= p, for a non-decreasing int array s with
-// s[0] = 0 <= p (the owner of item p in a load-balanced expansion)
-__device__ __forceinline__ int owner_of(const int* s, int n, int p) {
-    int lo = 0, len = n;
-    while (len > 0) {
-        int h = len >> 1;
-        if (s[lo + h] <= p) {
-            lo += h + 1;
-            len -= h + 1;
-        } else {
-            len = h;
-        }
-    }
-    return lo - 1;
-}
-
-// ---------------------------------------------------------------------------
 // block-wide exclusive scan of one int per thread; returns the exclusive
 // prefix, writes the block total.  `tmp` holds >= 33 ints of shared memory.
 // Contains __syncthreads(); every thread of the block must call it.
@@ -185,13 +135,13 @@ __device__ __forceinline__ int block_exscan(int v, int* tmp, int& total) {
 
 // The same scan with one barrier: every warp adds up the partial sums of the
 // warps before it itself.  Consecutive calls alternate between the two halves
-// of `buf` (>= 34 ints) under the block-uniform toggle `par`, so a call never
+// of `buf` (kScanInts ints) under the block-uniform toggle `par`, so a call never
 // overwrites partial sums that a slower thread may still read from the
 // previous call (the barrier of the call in between orders them).
 __device__ __forceinline__ int block_exscan1(int v, int* buf, int& par, int& total) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nw = (blockDim.x + 31) >> 5;
-    int* t = buf + (par ? 17 : 0);
+    int* t = buf + (par ? kScanInts / 2 : 0);
     par ^= 1;
     int x = v;
 #pragma unroll
@@ -212,12 +162,14 @@ __device__ __forceinline__ int block_exscan1(int v, int* buf, int& par, int& tot
     return x - v + before;
 }
 
-// block_exscan1 that also returns whether any thread's flag was set (the
-// flag rides in bit 30 of the warp partials; the values must stay below 2^30).
-__device__ __forceinline__ int block_exscan1_any(int v, bool flag, int* buf, int& par, int& total, bool& any) {
+// block_exscan1 that also ranks the threads with v > 0 (rank: how many before
+// this one; n_nz: how many in all).  nbuf holds kScanInts ints like buf.
+__device__ __forceinline__ int block_exscan1_nz(int v, int* buf, int* nbuf, int& par, int& total, int& rank,
+                                                int& n_nz) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nw = (blockDim.x + 31) >> 5;
-    int* t = buf + (par ? 17 : 0);
+    int* t = buf + (par ? kScanInts / 2 : 0);
+    int* u = nbuf + (par ? kScanInts / 2 : 0);
     par ^= 1;
     int x = v;
 #pragma unroll
@@ -225,21 +177,17 @@ __device__ __forceinline__ int block_exscan1_any(int v, bool flag, int* buf, int
         const int y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
     }
-    const int f = __any_sync(0xffffffffu, flag) ? (1 << 30) : 0;
-    if (lane == 31) t[wid] = x | f;
-    __syncthreads();
-    const int tw = lane < nw ? t[lane] : 0;
-    int w = tw & ((1 << 30) - 1);
-    int before = lane < wid ? w : 0;
-    const bool fa = __any_sync(0xffffffffu, (tw >> 30) & 1);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        w += __shfl_xor_sync(0xffffffffu, w, o);
-        before += __shfl_xor_sync(0xffffffffu, before, o);
+    const unsigned nz = __ballot_sync(0xffffffffu, v > 0);
+    if (lane == 31) {
+        t[wid] = x;
+        u[wid] = __popc(nz);
     }
-    total = w;
-    any = fa;
-    return x - v + before;
+    __syncthreads();
+    const int w = lane < nw ? t[lane] : 0, c = lane < nw ? u[lane] : 0;
+    total = __reduce_add_sync(0xffffffffu, w);
+    n_nz = __reduce_add_sync(0xffffffffu, c);
+    rank = __reduce_add_sync(0xffffffffu, lane < wid ? c : 0) + __popc(nz & ((1u << lane) - 1u));
+    return x - v + __reduce_add_sync(0xffffffffu, lane < wid ? w : 0);
 }
 
 __device__ __forceinline__ int warp_sum(int v) {

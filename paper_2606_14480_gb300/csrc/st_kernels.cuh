@@ -34,8 +34,7 @@ struct BuildArgs {
     int32_t* item_class;  // [2 n_events] cost class of each (event, half) seeding item
     int32_t* class_count; // [128] items per class, zero before the launch
     int32_t* class_fill;  // [128] places taken per class, zero before the launch
-    int32_t* order;       // [2 n_events] the seeding items, costliest class first
-    int32_t* zero2 = nullptr;  // [2 n_events] cleared by k_order (fused matching's counters), may be null
+    int32_t* order;       // [2 n_events] the seeding items, costliest class first; null: not needed
     int32_t* queue;
     unsigned long long* counters;
 };
@@ -51,6 +50,7 @@ struct SeedArgs {
     int32_t cand_cap;     // candidates per work item
     int32_t tbl_smem;     // clone table entries in shared memory
     int32_t key_smem;     // UV keys in shared memory
+    int32_t round_hits;   // T1 hits per round of the x-z search (at most the CTA's threads)
     uint8_t* slot;        // per-CTA scratch
     int64_t slot_stride;  // bytes per CTA
     int32_t max_xhits;    // size of the per-CTA clone table in scratch
@@ -63,7 +63,7 @@ struct SeedArgs {
     unsigned long long* pool_ctr;
     int32_t* item_start;
     int32_t* item_count;
-    const int32_t* order;  // the order k_build gave the items
+    const int32_t* order;  // the order of the items; null: each CTA has the one item of its own number
     int32_t* queue;
     unsigned long long* counters;
     // matching fused into the seeding kernel (velo null: seeding only): the
@@ -120,13 +120,24 @@ struct MatchArgs {
     float* chi2;
     int32_t* n_long;
     int32_t velo_smem;    // VELO segments per shared-memory chunk
-    int32_t* queue;
+    int32_t* queue;       // null: the grid covers the events
     unsigned long long* counters;
 };
+
+// The seeding kernel comes in CTAs of up to kSeedThreads[i] threads; its
+// instantiations are spread over translation units that compile in parallel.
+constexpr int kSeedShapes = 3;
+constexpr int kSeedThreads[kSeedShapes] = {256, 448, 512};
+typedef void (*SeedKernel)(const DevParams, const SeedArgs);
+// the instantiation for CTAs of `threads` threads, with the HLT2-style pass
+// loop (seq) or with the matching fused in
+SeedKernel seed_kernel(int threads, bool seq, bool fused);
 
 size_t build_smem_bytes(int bins, int smem_hits);
 size_t seed_smem_bytes(int threads, int smem_hits, int tbl_smem, int key_smem);
 size_t seed_slot_bytes(int cand_cap, int max_xhits);
+size_t seed_smem_limit_bytes(int threads, int smem_hits, int tbl_smem, int key_smem);
+size_t seed_slot_limit_bytes(int cand_cap, int max_xhits);
 size_t match_smem_bytes(int velo_smem);
 
 // chained: k_order, k_seed and k_scan are launched as programmatic dependents
@@ -136,7 +147,7 @@ size_t match_smem_bytes(int velo_smem);
 // stream's kernels want those SMs.
 cudaError_t launch_build(const DevParams& P, const BuildArgs& a, int grid, int threads, cudaStream_t s,
                          bool chained = true);
-cudaError_t launch_seed(const DevParams& P, const SeedArgs& a, int grid, int threads, cudaStream_t s,
+cudaError_t launch_seed(const DevParams& P, const SeedArgs& a, int grid, int threads, size_t smem, cudaStream_t s,
                         bool chained = true);
 cudaError_t launch_gather(const GatherArgs& a, cudaStream_t s, bool chained = true);
 cudaError_t launch_match(const DevParams& P, const MatchArgs& a, int grid, int threads, cudaStream_t s);
@@ -144,7 +155,7 @@ cudaError_t launch_match(const DevParams& P, const MatchArgs& a, int grid, int t
 // occupancy helpers
 int build_blocks_per_sm(int threads, size_t smem);
 int seed_blocks_per_sm(int threads, size_t smem);
-int match_blocks_per_sm(int threads, size_t smem);
+int match_blocks_per_sm(int threads, size_t smem, bool final_sel);
 cudaError_t set_smem_limits(size_t optin);
 cudaError_t smem_limits_hold(size_t optin, bool& hold);
 

@@ -314,9 +314,6 @@ bool derive_params(const st_config& c, DevParams& P, std::string& err) {
         const int u = uslot(c.uv_init[p]);
         if (u < 0) return fail("uv_init must name stereo layers");
         P.uv_init[p] = u;
-        int q = 0;
-        for (int v = 0; v < 6; ++v)
-            if (v != u) P.uv_rem[p][q++] = v;
     }
     P.n_uv_min = c.n_uv_min;
     P.uv_tol = static_cast<float>(c.uv_tol);
@@ -396,7 +393,7 @@ struct Workspace {
     int build_ctas = 0, seed_ctas = 0;  // CTAs the per-CTA scratch is sized for
     // carved pointers
     // [0] build, [1] seed, [2] match queues; fused matching: [3] announced, [4] fault,
-    // [5] claimed, [6] done; [16, 144) item classes, [144, 272) their fill
+    // [5] claimed, [6] done; [16, 144) item classes, [144, 272) their fill; then ev_done
     int32_t* queues = nullptr;
     unsigned long long* pool_ctr = nullptr;
     float* cx = nullptr;
@@ -421,6 +418,14 @@ struct Workspace {
 
 struct Pipeline;
 
+// CTAs of the seeding kernel: threads, what their shared memory holds, and how
+// many an SM takes.
+struct SeedShape {
+    int threads = 0, smem_hits = 0, tbl_smem = 0, key_smem = 0, velo_smem = 0;
+    size_t smem = 0;
+    int bps = 0;
+};
+
 constexpr int64_t kDefaultWaitNs = 200000000;  // 200 ms
 
 struct st_ctx {
@@ -432,9 +437,11 @@ struct st_ctx {
     std::string err;
     unsigned long long* counters = nullptr;
     Workspace ws;
-    int tbl_smem = 0, key_smem = 0, velo_smem = 0;
-    size_t seed_smem = 0, match_smem = 0, build_smem_max = 0;
-    int seed_bps = 0, match_bps = 0;
+    int velo_smem = 0;
+    size_t match_smem = 0, build_smem_max = 0;
+    SeedShape shape[kSeedShapes];  // [0] as configured, then the larger CTAs for batches that leave SMs idle
+    int n_shapes = 0;
+    int match_bps = 0;
     Pipeline* pipe = nullptr;
     std::mutex pipe_mu;
     bool timing = false;
@@ -505,9 +512,9 @@ static size_t carve(st_ctx* ctx, Workspace& w, int64_t ne, int64_t nh, int32_t m
         return base ? base + o : nullptr;
     };
     const int build_ctas = ctx->n_sms * kBuildCtasPerSm;
-    const int seed_ctas = ctx->n_sms * std::max(1, ctx->seed_bps);
+    const int seed_ctas = ctx->n_sms * std::max(1, ctx->shape[0].bps);
     const int64_t items = 2 * ne;
-    char* q = take(kQueueBytes);
+    char* q = take(kQueueBytes + sizeof(int32_t) * size_t(items));  // zeroed per launch as one range
     char* cx = take(sizeof(float) * size_t(nh + 3 * ne + 8));
     char* co = take(sizeof(int32_t) * size_t(nh + 3 * ne + 8));
     char* zo = take(sizeof(int32_t) * size_t(ne) * kZoffStride + 4);
@@ -523,7 +530,6 @@ static size_t carve(st_ctx* ctx, Workspace& w, int64_t ne, int64_t nh, int32_t m
     char* ic = take(sizeof(int32_t) * size_t(items) + 4);
     char* icl = take(sizeof(int32_t) * size_t(items) + 4);
     char* ord = take(sizeof(int32_t) * size_t(items) + 4);
-    char* evd = take(sizeof(int32_t) * size_t(items) + 4);
     char* pv = take(sizeof(int32_t) * size_t(sc) + 4);
     char* pc = take(sizeof(float) * size_t(sc) + 4);
     if (base) {
@@ -544,7 +550,7 @@ static size_t carve(st_ctx* ctx, Workspace& w, int64_t ne, int64_t nh, int32_t m
         w.item_count = reinterpret_cast<int32_t*>(ic);
         w.item_class = reinterpret_cast<int32_t*>(icl);
         w.order = reinterpret_cast<int32_t*>(ord);
-        w.ev_done = reinterpret_cast<int32_t*>(evd);
+        w.ev_done = reinterpret_cast<int32_t*>(q + kQueueBytes);
         w.pool_velo = reinterpret_cast<int32_t*>(pv);
         w.pool_chi2 = reinterpret_cast<float*>(pc);
         w.cap_events = ne;
@@ -609,14 +615,24 @@ extern "C" int st_create(const st_config* cfg, int device, st_ctx** out) {
     }
     ctx->smem_optin = optin;
     const st_config& c = *cfg;
-    ctx->tbl_smem = c.smem_hits / 2;
-    ctx->key_smem = std::max(64, c.smem_hits / 8);  // kept seeds whose UV keys and stereo x stay in shared memory
+    auto add_shape = [&](int threads, int smem_hits, int velo_smem) {
+        SeedShape& s = ctx->shape[ctx->n_shapes++];
+        s.threads = threads;
+        s.smem_hits = smem_hits;
+        s.tbl_smem = smem_hits / 2;
+        s.key_smem = std::max(64, smem_hits / 8);  // kept seeds whose UV keys and stereo x stay in shared memory
+        s.velo_smem = velo_smem;
+        s.smem = std::max(seed_smem_bytes(threads, smem_hits, s.tbl_smem, s.key_smem), match_smem_bytes(velo_smem));
+    };
+    add_shape(c.threads_seed, c.smem_hits, 512);
     ctx->velo_smem = 512;
-    ctx->seed_smem = seed_smem_bytes(c.threads_seed, c.smem_hits, ctx->tbl_smem, ctx->key_smem);
     ctx->match_smem = match_smem_bytes(ctx->velo_smem);
     ctx->build_smem_max = build_smem_bytes(512, kBuildSmemHits);
     // 2 KB of margin for the kernels' static shared memory
-    if (ctx->seed_smem + 2048 > ctx->smem_optin || ctx->build_smem_max + 2048 > ctx->smem_optin) {
+    const SeedShape& s0 = ctx->shape[0];
+    const size_t seed_limit =
+        std::max(s0.smem, seed_smem_limit_bytes(c.threads_seed, c.smem_hits, s0.tbl_smem, s0.key_smem));
+    if (seed_limit + 2048 > ctx->smem_optin || ctx->build_smem_max + 2048 > ctx->smem_optin) {
         delete ctx;
         return ST_EINVAL;
     }
@@ -630,8 +646,10 @@ extern "C" int st_create(const st_config* cfg, int device, st_ctx** out) {
         delete ctx;
         return ST_ECUDA;
     }
-    ctx->seed_bps = seed_blocks_per_sm(c.threads_seed, ctx->seed_smem);
-    ctx->match_bps = match_blocks_per_sm(c.threads_match, ctx->match_smem);
+    if (c.threads_seed < 448) add_shape(448, 2048, 768);
+    if (c.threads_seed < 512) add_shape(512, 4096, 1024);
+    for (int k = 0; k < ctx->n_shapes; ++k) ctx->shape[k].bps = seed_blocks_per_sm(ctx->shape[k].threads, ctx->shape[k].smem);
+    ctx->match_bps = match_blocks_per_sm(c.threads_match, ctx->match_smem, c.final_sel != 0);
     *out = ctx;
     return ST_OK;
 }
@@ -667,6 +685,20 @@ extern "C" int st_reserve(st_ctx* ctx, int64_t n_events, int64_t n_hits, int32_t
 // seeding / matching
 // ---------------------------------------------------------------------------
 
+// The seeding CTAs for a batch of so many (event, half) items: the largest
+// CTAs that take it in one round.  Such a batch is bound by the latency of one
+// item, which falls with the threads that share it; above that the SMs are
+// shared anyway and the smaller CTAs pass their barriers sooner.  k_seed,
+// Run-3-like events, at 256 / 448 / 512 threads: 67 events 69 / 57 / 53 us, 150
+// events 90 / 71 / 65, 220 events 91 / 81 / 85, 300 events 91 / 96 / 95, 1000
+// events 191 / 233 / 271.  A set ctas_per_sm asks for the configured shape.
+static const SeedShape& seed_shape(const st_ctx* ctx, int64_t items) {
+    if (ctx->cfg.ctas_per_sm > 0) return ctx->shape[0];
+    for (int k = ctx->n_shapes - 1; k > 0; --k)
+        if (items <= int64_t(ctx->n_sms) * ctx->shape[k].bps) return ctx->shape[k];
+    return ctx->shape[0];
+}
+
 // With V and L (fused): the seeding kernel also matches each event once its
 // two halves are done, and the gather writes the Long tracks too.
 static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S, cudaStream_t s,
@@ -681,16 +713,19 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
     if (c.ctas_per_sm > 0) bbps = std::min(bbps, c.ctas_per_sm);
     const int g_build = static_cast<int>(std::max<int64_t>(
         1, std::min<int64_t>({H.n_events, int64_t(ctx->n_sms) * bbps, int64_t(w.build_ctas)})));
-    int sbps = std::max(1, ctx->seed_bps);
+    const SeedShape& sh = seed_shape(ctx, 2 * H.n_events);
+    int sbps = std::max(1, sh.bps);
     if (c.ctas_per_sm > 0) sbps = std::min(sbps, c.ctas_per_sm);
     const int g_seed = static_cast<int>(std::max<int64_t>(
         1, std::min<int64_t>({2 * H.n_events, int64_t(ctx->n_sms) * sbps, int64_t(w.seed_ctas)})));
-    ST_CUDA(ctx, cudaMemsetAsync(w.queues, 0, kQueueBytes, s));
+    const bool fused = V && L;
+    ST_CUDA(ctx, cudaMemsetAsync(w.queues, 0, kQueueBytes + (fused ? 2 * sizeof(int32_t) * size_t(H.n_events) : 0), s));
     if (H.n_events == 0) {
         ST_CUDA(ctx, cudaMemsetAsync(S.ev_off, 0, sizeof(int32_t), s));
         return ST_OK;
     }
-    const bool fused = V && L;
+    // every item has a CTA of its own from the start: no queue, no order
+    const bool one_round = 2 * H.n_events <= g_seed;
     BuildArgs b;
     b.n_events = H.n_events;
     b.ev_off = H.ev_off;
@@ -711,8 +746,7 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
     b.item_class = w.item_class;
     b.class_count = w.queues + 16;
     b.class_fill = w.queues + 16 + 128;
-    b.order = w.order;
-    b.zero2 = fused ? w.ev_done : nullptr;  // halves done + announcements, cleared before k_seed
+    b.order = one_round ? nullptr : w.order;
     b.queue = w.queues + 0;
     b.counters = ctx->counters;
     // k_order, the seeding kernel and the scan follow their predecessors as
@@ -734,10 +768,11 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
     a.corig = w.corig;
     a.zoff = w.zoff;
     a.status = S.status;
-    a.smem_hits = ctx->cfg.smem_hits;
+    a.smem_hits = sh.smem_hits;
     a.cand_cap = ctx->cfg.cand_cap;
-    a.tbl_smem = ctx->tbl_smem;
-    a.key_smem = ctx->key_smem;
+    a.tbl_smem = sh.tbl_smem;
+    a.key_smem = sh.key_smem;
+    a.round_hits = c.threads_seed;
     a.slot = w.slot;
     a.slot_stride = w.slot_stride;
     a.max_xhits = w.cap_max_hits;
@@ -749,15 +784,19 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
     a.pool_ctr = w.pool_ctr;
     a.item_start = w.item_start;
     a.item_count = w.item_count;
-    a.order = w.order;
+    a.order = b.order;
     a.queue = w.queues + 1;
     a.counters = ctx->counters;
     a.fault = w.queues + 4;  // a wait that gave up (staging copy, announced event)
     if (fused) {
         a.velo_off = V->ev_off;
         a.velo = V->state;
-        a.velo_smem = ctx->velo_smem;
-        a.defer_match = defer ? 1 : 0;
+        a.velo_smem = sh.velo_smem;
+        // Matching the last events where a CTA is free evens out the CTAs'
+        // finishing times; with one item each there is nothing to even out, and
+        // the waiting CTAs slow the others down (250 Run-3-like events: 117 us
+        // with it, 107 without).  A wait limit of 0 asks for the waits' timeout.
+        a.defer_match = defer && (!one_round || ctx->wait_ns == 0) ? 1 : 0;
         a.ev_done = w.ev_done;
         a.ready = w.ev_done + H.n_events;
         a.ready_ctr = w.queues + 3;
@@ -770,7 +809,7 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
         if (ctx->timing && &w == &ctx->ws) ctx->tused[3] = false;  // matching runs inside k_seed
     }
     tmark(ctx, w, 1, 0, s);
-    ST_CUDA(ctx, launch_seed(ctx->P, a, g_seed, c.threads_seed, s, chain && !marks));
+    ST_CUDA(ctx, launch_seed(ctx->P, a, g_seed, sh.threads, sh.smem, s, chain && !marks));
     tmark(ctx, w, 1, 1, s);
 
     GatherArgs g;
@@ -805,7 +844,6 @@ static int run_matching(st_ctx* ctx, Workspace& w, const st_velo& V, const st_se
                         cudaStream_t s) {
     if (V.n_events == 0) return ST_OK;
     if (!w.base) return set_err(ctx, ST_ESTATE, "matching_run before any seeding_run on this context");
-    ST_CUDA(ctx, cudaMemsetAsync(w.queues + 2, 0, sizeof(int32_t), s));
     MatchArgs m;
     m.n_events = V.n_events;
     m.velo_off = V.ev_off;
@@ -822,11 +860,15 @@ static int run_matching(st_ctx* ctx, Workspace& w, const st_velo& V, const st_se
     m.seed_n = S.n_hits;
     m.ghost_prob = L.ghost_prob;
     m.velo_smem = ctx->velo_smem;
-    m.queue = w.queues + 2;
     m.counters = ctx->counters;
     int mbps = std::max(1, ctx->match_bps);
     if (ctx->cfg.ctas_per_sm > 0) mbps = std::min(mbps, ctx->cfg.ctas_per_sm);
     const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(V.n_events, int64_t(ctx->n_sms) * mbps)));
+    m.queue = nullptr;
+    if (grid < V.n_events) {
+        m.queue = w.queues + 2;
+        ST_CUDA(ctx, cudaMemsetAsync(m.queue, 0, sizeof(int32_t), s));
+    }
     tmark(ctx, w, 3, 0, s);
     ST_CUDA(ctx, launch_match(ctx->P, m, grid, ctx->cfg.threads_match, s));
     tmark(ctx, w, 3, 1, s);
@@ -834,12 +876,11 @@ static int run_matching(st_ctx* ctx, Workspace& w, const st_velo& V, const st_se
 }
 
 // Seeding then matching of one batch.  The fused kernel (matching inside the
-// seeding kernel) serves the HLT1 configuration with 256-thread seeding CTAs
-// and no final selection; every other configuration runs the two steps apart.
+// seeding kernel) serves the HLT1 configuration without the final selection;
+// every other configuration runs the two steps apart.
 static bool fusable(const st_ctx* ctx, const st_hits& H, const st_velo& V) {
     const st_config& c = ctx->cfg;
-    return c.threads_seed <= 256 && c.iter_mode == 0 && !c.final_sel && V.n_events == H.n_events &&
-           match_smem_bytes(ctx->velo_smem) <= ctx->seed_smem;
+    return c.iter_mode == 0 && !c.final_sel && V.n_events == H.n_events;
 }
 
 // defer: the kernel has the GPU to itself (a graph replay), so CTAs without

@@ -1,0 +1,32 @@
+// st_seed.cu -- sizes of the seeding kernel's memory and the choice of its
+// instantiation.
+#include "st_seed.cuh"
+
+namespace st {
+
+size_t seed_smem_bytes(int threads, int smem_hits, int tbl_smem, int key_smem) {
+    return seed_smem_size(threads, smem_hits, tbl_smem, key_smem);
+}
+size_t seed_slot_bytes(int cand_cap, int max_xhits) { return seed_slot_size(cand_cap, max_xhits); }
+
+// The shared memory and the scratch per CTA that a configuration is accepted
+// by (no less than what the kernel takes of either): what the interface's
+// limits are stated in.
+size_t seed_smem_limit_bytes(int threads, int smem_hits, int tbl_smem, int key_smem) {
+    return align16(sizeof(float) * smem_hits) + 9216 + sizeof(ull) * (tbl_smem + key_smem) +
+           sizeof(float) * 6 * key_smem + sizeof(int) * 3 * threads + sizeof(int) * (36 + 16);
+}
+size_t seed_slot_limit_bytes(int cand_cap, int max_xhits) {
+    return align16(sizeof(int) * 16 * size_t(cand_cap)) +
+           sizeof(ull) * (size_t(max_xhits) + cand_cap + size_t(kTripPerCand) * cand_cap) +
+           16 + (2 * sizeof(uint4) + sizeof(uint2)) * kUvStore + sizeof(float) * 6 * size_t(cand_cap) + 8 +
+           sizeof(ull) * 12 * 512 + 9 * size_t(cand_cap) + 4 + sizeof(uint32_t) * ((size_t(max_xhits) + 31) / 32);
+}
+
+SeedKernel seed_kernel(int threads, bool seq, bool fused) {
+    return threads <= 256 ? seed_kernel_256(seq, fused)
+           : threads <= 448 ? seed_kernel_448(seq, fused)
+                            : seed_kernel_512(seq, fused);
+}
+
+}  // namespace st

@@ -141,12 +141,14 @@ extern "C" int seeding_run_static(const st_config* cfg, const st_hits* H, st_see
     const size_t o_ps = take(sizeof(float) * 4 * size_t(S->cap) + 4);
     const size_t o_pn = take(2 * size_t(S->cap) + 4);
     const size_t slot_stride = up256(seed_slot_bytes(cfg->cand_cap, static_cast<int>(mh)));
+    const size_t slot_limit =
+        std::max(slot_stride, up256(seed_slot_limit_bytes(cfg->cand_cap, static_cast<int>(mh))));
     const size_t fixed = off;
-    if (fixed + slot_stride > size_t(ST_STATIC_SCRATCH_BYTES))
+    if (fixed + slot_limit > size_t(ST_STATIC_SCRATCH_BYTES))
         return fail(err, err_len, ST_OVERFLOW,
                     "batch needs %zu bytes of scratch (%lld events, max %lld hits/event, %lld seeds) but the "
                     "static scratch holds %zu; split the batch or lower seeds cap / cand_cap",
-                    fixed + slot_stride, (long long)ne, (long long)mh, (long long)S->cap,
+                    fixed + slot_limit, (long long)ne, (long long)mh, (long long)S->cap,
                     size_t(ST_STATIC_SCRATCH_BYTES));
     const int64_t slots_fit = int64_t((size_t(ST_STATIC_SCRATCH_BYTES) - fixed) / slot_stride);
     unsigned char* b = D->base;
@@ -169,10 +171,12 @@ extern "C" int seeding_run_static(const st_config* cfg, const st_hits* H, st_see
     const int tbl_smem = cfg->smem_hits / 2, key_smem = std::max(64, cfg->smem_hits / 8);  // as st_create
     const size_t ssmem = seed_smem_bytes(cfg->threads_seed, cfg->smem_hits, tbl_smem, key_smem);
     // the shared-memory check of st_create (2 KB left for static shared memory)
-    if (ssmem + 2048 > size_t(D->optin) || bsmem + 2048 > size_t(D->optin))
+    const size_t slimit =
+        std::max(ssmem, seed_smem_limit_bytes(cfg->threads_seed, cfg->smem_hits, tbl_smem, key_smem));
+    if (slimit + 2048 > size_t(D->optin) || bsmem + 2048 > size_t(D->optin))
         return fail(err, err_len, ST_EINVAL,
                     "config needs %zu (seeding) / %zu (containers) bytes of shared memory per CTA; the device "
-                    "allows %d", ssmem, bsmem, D->optin);
+                    "allows %d", slimit, bsmem, D->optin);
     int bbps = std::max(1, build_blocks_per_sm(cfg->threads_build, bsmem));
     int sbps = std::max(1, seed_blocks_per_sm(cfg->threads_seed, ssmem));
     if (cfg->ctas_per_sm > 0) {  // as seeding_run
@@ -203,7 +207,7 @@ extern "C" int seeding_run_static(const st_config* cfg, const st_hits* H, st_see
     ba.item_class = reinterpret_cast<int32_t*>(b + o_icl);
     ba.class_count = queues + 16;
     ba.class_fill = queues + 16 + 128;
-    ba.order = reinterpret_cast<int32_t*>(b + o_ord);
+    ba.order = items <= g_seed ? nullptr : reinterpret_cast<int32_t*>(b + o_ord);
     ba.queue = queues + 0;
     ba.counters = counters;
     e = launch_build(P, ba, g_build, cfg->threads_build, s);
@@ -220,6 +224,7 @@ extern "C" int seeding_run_static(const st_config* cfg, const st_hits* H, st_see
     sa.cand_cap = cfg->cand_cap;
     sa.tbl_smem = tbl_smem;
     sa.key_smem = key_smem;
+    sa.round_hits = cfg->threads_seed;
     sa.slot = b + fixed;
     sa.slot_stride = static_cast<int64_t>(slot_stride);
     sa.max_xhits = static_cast<int32_t>(mh);
@@ -235,7 +240,7 @@ extern "C" int seeding_run_static(const st_config* cfg, const st_hits* H, st_see
     sa.queue = queues + 1;
     sa.counters = counters;
     sa.fault = queues + 4;  // set if a staging copy was given up on
-    e = launch_seed(P, sa, g_seed, cfg->threads_seed, s);
+    e = launch_seed(P, sa, g_seed, cfg->threads_seed, ssmem, s);
     if (e != cudaSuccess) return fail(err, err_len, ST_ECUDA, "k_seed: %s", cudaGetErrorString(e));
 
     GatherArgs ga;

@@ -1,0 +1,74 @@
+"""The block-wide walk of the seeding kernel at its edges.
+
+Pairs are walked in groups of 32 and blocks of 12 groups per warp, triplets
+wait in queues of 128 per warp, UV combinations go in blocks of 1024, and
+batches of up to two items per SM run in larger CTAs.  Wide third-hit bands and
+windows, tiny events and batch sizes around that limit reach every branch; the
+oracle, and the same batch in CTAs of other sizes, say what is right."""
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import parity  # noqa: E402
+from conftest import workload  # noqa: E402
+from paper_2606_14480_gb300 import st  # noqa: E402
+from synth import calibrate_zmatch, make_events  # noqa: E402
+from test_gpu_parity import run_gpu  # noqa: E402
+
+KEYS = ("ev_off", "hits", "params", "state", "n_hits", "status", "velo_idx", "chi2", "n_long")
+
+
+@pytest.fixture(scope="module")
+def zmx():
+    return calibrate_zmatch(7826.0)
+
+
+def run(b, zmx, **over):
+    _, gcfg = parity.config_pair(zmx, **over)
+    ctx = st.Context(gcfg)
+    out = st.run_batch(ctx, st.DeviceBatch.from_synth(b)).to_numpy()
+    ctx.close()
+    return out
+
+
+@pytest.mark.parametrize("n,tracks,over", [
+    (6, 400, dict(m_lo=0.0, m_hi=40.0, cand_cap=65536)),                     # queues of triplets run over
+    (2, 200, dict(m_lo=0.0, m_hi=400.0, chi2x_max=0.5, cand_cap=65536)),     # single groups hold more than a queue
+    (6, 300, dict(uv_y_overlap=2500.0, n_uv_min=3)),                         # blocks of UV combinations
+    (40, 1, {}), (40, 3, dict(n_uv_min=2)),                                  # less than a warp of anything
+])
+def test_walk_edges_parity_and_shapes(n, tracks, over, zmx):
+    b = make_events(n, seed=4001, tracks=("fixed", tracks))
+    ocfg, gcfg = parity.config_pair(zmx, **over)
+    gpu, _ = run_gpu(b, gcfg)
+    assert (gpu["status"] == 0).all()
+    # the harness's bars, except that on chi2: wide bands make combinations
+    # whose chi2 is far below the default band's, where its relative error says
+    # nothing about the walk
+    rep = parity.compare_seeding(gpu, ocfg, b)
+    assert rep.agreement >= parity.AGREE_MIN and not rep.untraced and not rep.bad_params, rep.summary()
+    for shape in (dict(threads_seed=64), dict(threads_seed=96, ctas_per_sm=1), dict(threads_seed=256, ctas_per_sm=8)):
+        other = run(b, zmx, **over, **shape)
+        for k in ("ev_off", "hits", "params", "state"):
+            assert np.array_equal(other[k], gpu[k]), (shape, k)
+
+
+@pytest.mark.parametrize("mode", [{}, dict(uv_mode=1), dict(iter_mode=1)], ids=["hlt1", "hough", "seq"])
+def test_larger_ctas_give_the_same(mode, zmx):
+    """Around the largest batch that the larger CTAs take in one round: every
+    event's result is that of the batch one event larger."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    b = workload("run3", n_events=sms + 1)
+    big = run(b, zmx, **mode)
+    small = run(b.subset(range(sms)), zmx, **mode)
+    n = small["ev_off"][-1]
+    assert np.array_equal(small["ev_off"], big["ev_off"][:-1]) and (big["status"] == 0).all()
+    for k in KEYS[1:]:
+        assert np.array_equal(small[k], big[k][:len(small[k])]), k
+    assert n > 0
