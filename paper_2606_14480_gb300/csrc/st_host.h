@@ -5,9 +5,29 @@
 
 #include "st.h"
 #include "st_device.cuh"
+#include "st_kernels.cuh"
 
 namespace st {
-}
+
+// CTAs of the seeding kernel: threads, what their shared memory holds, and how
+// many an SM takes.
+struct SeedShape {
+    int threads = 0, smem_hits = 0, tbl_smem = 0, key_smem = 0, velo_smem = 0;
+    size_t smem = 0;
+    int bps = 0;
+};
+
+// The shapes a configuration may run with: [0] as configured, then larger CTAs
+// for batches that leave SMs idle.  Returns how many; with `bps`, how many CTAs
+// of each an SM takes (after set_smem_limits).
+int seed_shapes(const st_config& c, SeedShape out[kSeedShapes], bool bps);
+
+// The shape for a batch of `items` (event, half) items when at most `max_ctas`
+// CTAs may run (their scratch).
+const SeedShape& pick_seed_shape(const SeedShape* shapes, int n, const st_config& c, int64_t items, int n_sms,
+                                 int64_t max_ctas);
+
+}  // namespace st
 
 // Derive the device constants from a configuration (validates it; false and a
 // message on an invalid configuration).

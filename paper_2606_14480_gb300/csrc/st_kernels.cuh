@@ -53,7 +53,8 @@ struct SeedArgs {
     int32_t round_hits;   // T1 hits per round of the x-z search (at most the CTA's threads)
     uint8_t* slot;        // per-CTA scratch
     int64_t slot_stride;  // bytes per CTA
-    int32_t max_xhits;    // size of the per-CTA clone table in scratch
+    int32_t uv_cap;       // valid UV combinations stored per work item (at most kUvStore)
+    int32_t tbl_cap;      // clone table entries in scratch (for halves above tbl_smem)
     // staging pool of seed records
     int32_t* pool_hits;
     float* pool_params;
@@ -64,6 +65,11 @@ struct SeedArgs {
     int32_t* item_start;
     int32_t* item_count;
     const int32_t* order;  // the order of the items; null: each CTA has the one item of its own number
+    const int32_t* n_list = nullptr;  // on the device: items in `order`; null: 2 n_events
+    // items that need more scratch than a CTA has are listed here for a launch
+    // with more; null: their events get ST_OVERFLOW
+    int32_t* retry = nullptr;
+    int32_t* retry_ctr = nullptr;
     int32_t* queue;
     unsigned long long* counters;
     // matching fused into the seeding kernel (velo null: seeding only): the
@@ -135,7 +141,8 @@ SeedKernel seed_kernel(int threads, bool seq, bool fused);
 
 size_t build_smem_bytes(int bins, int smem_hits);
 size_t seed_smem_bytes(int threads, int smem_hits, int tbl_smem, int key_smem);
-size_t seed_slot_bytes(int cand_cap, int max_xhits);
+constexpr int kUvStore = 8191;  // most valid UV combinations stored per work item
+size_t seed_slot_bytes(int cand_cap, int uv_cap, int tbl_cap, int max_hits);
 size_t seed_smem_limit_bytes(int threads, int smem_hits, int tbl_smem, int key_smem);
 size_t seed_slot_limit_bytes(int cand_cap, int max_xhits);
 size_t match_smem_bytes(int velo_smem);

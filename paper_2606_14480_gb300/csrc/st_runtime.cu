@@ -381,6 +381,47 @@ bool derive_params(const st_config& c, DevParams& P, std::string& err) {
 }
 
 // ---------------------------------------------------------------------------
+// shapes of the seeding kernel
+// ---------------------------------------------------------------------------
+
+namespace st {
+
+int seed_shapes(const st_config& c, SeedShape out[kSeedShapes], bool bps) {
+    int n = 0;
+    auto add = [&](int threads, int smem_hits, int velo_smem) {
+        SeedShape& s = out[n++];
+        s.threads = threads;
+        s.smem_hits = smem_hits;
+        s.tbl_smem = smem_hits / 2;
+        s.key_smem = std::max(64, smem_hits / 8);  // kept seeds whose UV keys and stereo x stay in shared memory
+        s.velo_smem = velo_smem;
+        s.smem = std::max(seed_smem_bytes(threads, smem_hits, s.tbl_smem, s.key_smem), match_smem_bytes(velo_smem));
+        s.bps = bps ? seed_blocks_per_sm(threads, s.smem) : 0;
+    };
+    add(c.threads_seed, c.smem_hits, 512);
+    if (c.threads_seed < 448) add(448, 2048, 768);
+    if (c.threads_seed < 512) add(512, 4096, 1024);
+    return n;
+}
+
+// The largest CTAs that take the batch in one round.  Such a batch is bound by
+// the latency of one item, which falls with the threads that share it; above
+// that the SMs are shared anyway and the smaller CTAs pass their barriers
+// sooner.  k_seed, Run-3-like events, at 256 / 448 / 512 threads: 67 events 69 /
+// 57 / 53 us, 150 events 90 / 71 / 65, 220 events 91 / 81 / 85, 300 events 91 /
+// 96 / 95, 1000 events 191 / 233 / 271.  A set ctas_per_sm asks for the
+// configured shape.
+const SeedShape& pick_seed_shape(const SeedShape* shapes, int n, const st_config& c, int64_t items, int n_sms,
+                                 int64_t max_ctas) {
+    if (c.ctas_per_sm == 0)
+        for (int k = n - 1; k > 0; --k)
+            if (items <= std::min<int64_t>(int64_t(n_sms) * shapes[k].bps, max_ctas)) return shapes[k];
+    return shapes[0];
+}
+
+}  // namespace st
+
+// ---------------------------------------------------------------------------
 // workspace: one scratch arena and its launch shapes
 // ---------------------------------------------------------------------------
 
@@ -417,14 +458,6 @@ struct Workspace {
 };
 
 struct Pipeline;
-
-// CTAs of the seeding kernel: threads, what their shared memory holds, and how
-// many an SM takes.
-struct SeedShape {
-    int threads = 0, smem_hits = 0, tbl_smem = 0, key_smem = 0, velo_smem = 0;
-    size_t smem = 0;
-    int bps = 0;
-};
 
 constexpr int64_t kDefaultWaitNs = 200000000;  // 200 ms
 
@@ -520,7 +553,7 @@ static size_t carve(st_ctx* ctx, Workspace& w, int64_t ne, int64_t nh, int32_t m
     char* zo = take(sizeof(int32_t) * size_t(ne) * kZoffStride + 4);
     const int64_t big_stride = mh > kBuildSmemHits ? int64_t(al256(size_t(10) * mh)) : 0;
     char* big = take(size_t(big_stride) * build_ctas + 16);
-    const int64_t slot_stride = int64_t(al256(seed_slot_bytes(ctx->cfg.cand_cap, mh)));
+    const int64_t slot_stride = int64_t(al256(seed_slot_bytes(ctx->cfg.cand_cap, kUvStore, mh, mh)));
     char* slot = take(size_t(slot_stride) * seed_ctas);
     char* ph = take(sizeof(int32_t) * 12 * size_t(sc) + 4);
     char* pp = take(sizeof(float) * 8 * size_t(sc) + 4);
@@ -615,16 +648,7 @@ extern "C" int st_create(const st_config* cfg, int device, st_ctx** out) {
     }
     ctx->smem_optin = optin;
     const st_config& c = *cfg;
-    auto add_shape = [&](int threads, int smem_hits, int velo_smem) {
-        SeedShape& s = ctx->shape[ctx->n_shapes++];
-        s.threads = threads;
-        s.smem_hits = smem_hits;
-        s.tbl_smem = smem_hits / 2;
-        s.key_smem = std::max(64, smem_hits / 8);  // kept seeds whose UV keys and stereo x stay in shared memory
-        s.velo_smem = velo_smem;
-        s.smem = std::max(seed_smem_bytes(threads, smem_hits, s.tbl_smem, s.key_smem), match_smem_bytes(velo_smem));
-    };
-    add_shape(c.threads_seed, c.smem_hits, 512);
+    ctx->n_shapes = seed_shapes(c, ctx->shape, false);
     ctx->velo_smem = 512;
     ctx->match_smem = match_smem_bytes(ctx->velo_smem);
     ctx->build_smem_max = build_smem_bytes(512, kBuildSmemHits);
@@ -646,9 +670,7 @@ extern "C" int st_create(const st_config* cfg, int device, st_ctx** out) {
         delete ctx;
         return ST_ECUDA;
     }
-    if (c.threads_seed < 448) add_shape(448, 2048, 768);
-    if (c.threads_seed < 512) add_shape(512, 4096, 1024);
-    for (int k = 0; k < ctx->n_shapes; ++k) ctx->shape[k].bps = seed_blocks_per_sm(ctx->shape[k].threads, ctx->shape[k].smem);
+    ctx->n_shapes = seed_shapes(c, ctx->shape, true);
     ctx->match_bps = match_blocks_per_sm(c.threads_match, ctx->match_smem, c.final_sel != 0);
     *out = ctx;
     return ST_OK;
@@ -685,20 +707,6 @@ extern "C" int st_reserve(st_ctx* ctx, int64_t n_events, int64_t n_hits, int32_t
 // seeding / matching
 // ---------------------------------------------------------------------------
 
-// The seeding CTAs for a batch of so many (event, half) items: the largest
-// CTAs that take it in one round.  Such a batch is bound by the latency of one
-// item, which falls with the threads that share it; above that the SMs are
-// shared anyway and the smaller CTAs pass their barriers sooner.  k_seed,
-// Run-3-like events, at 256 / 448 / 512 threads: 67 events 69 / 57 / 53 us, 150
-// events 90 / 71 / 65, 220 events 91 / 81 / 85, 300 events 91 / 96 / 95, 1000
-// events 191 / 233 / 271.  A set ctas_per_sm asks for the configured shape.
-static const SeedShape& seed_shape(const st_ctx* ctx, int64_t items) {
-    if (ctx->cfg.ctas_per_sm > 0) return ctx->shape[0];
-    for (int k = ctx->n_shapes - 1; k > 0; --k)
-        if (items <= int64_t(ctx->n_sms) * ctx->shape[k].bps) return ctx->shape[k];
-    return ctx->shape[0];
-}
-
 // With V and L (fused): the seeding kernel also matches each event once its
 // two halves are done, and the gather writes the Long tracks too.
 static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S, cudaStream_t s,
@@ -713,7 +721,7 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
     if (c.ctas_per_sm > 0) bbps = std::min(bbps, c.ctas_per_sm);
     const int g_build = static_cast<int>(std::max<int64_t>(
         1, std::min<int64_t>({H.n_events, int64_t(ctx->n_sms) * bbps, int64_t(w.build_ctas)})));
-    const SeedShape& sh = seed_shape(ctx, 2 * H.n_events);
+    const SeedShape& sh = pick_seed_shape(ctx->shape, ctx->n_shapes, c, 2 * H.n_events, ctx->n_sms, w.seed_ctas);
     int sbps = std::max(1, sh.bps);
     if (c.ctas_per_sm > 0) sbps = std::min(sbps, c.ctas_per_sm);
     const int g_seed = static_cast<int>(std::max<int64_t>(
@@ -775,7 +783,8 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
     a.round_hits = c.threads_seed;
     a.slot = w.slot;
     a.slot_stride = w.slot_stride;
-    a.max_xhits = w.cap_max_hits;
+    a.uv_cap = kUvStore;
+    a.tbl_cap = w.cap_max_hits;
     a.pool_hits = w.pool_hits;
     a.pool_params = w.pool_params;
     a.pool_state = w.pool_state;

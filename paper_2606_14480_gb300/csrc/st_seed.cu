@@ -7,7 +7,9 @@ namespace st {
 size_t seed_smem_bytes(int threads, int smem_hits, int tbl_smem, int key_smem) {
     return seed_smem_size(threads, smem_hits, tbl_smem, key_smem);
 }
-size_t seed_slot_bytes(int cand_cap, int max_xhits) { return seed_slot_size(cand_cap, max_xhits); }
+size_t seed_slot_bytes(int cand_cap, int uv_cap, int tbl_cap, int max_hits) {
+    return seed_slot_size(cand_cap, uv_cap, tbl_cap, max_hits);
+}
 
 // The shared memory and the scratch per CTA that a configuration is accepted
 // by (no less than what the kernel takes of either): what the interface's

@@ -470,7 +470,6 @@ static __device__ void uv_fit(const DevParams& P, const float* X, const float* t
 // then pass A, then the earlier initial hit (the order of Section 3.4's
 // choice); the lowest 13 bits carry where the combination's hits were stored
 // (kUvNotStored if they were not) and never decide.
-constexpr int kUvStore = 8191;
 constexpr int kUvNotStored = 8191;
 
 __device__ __forceinline__ ull uv_key(int n, float chi2, int pass, int kinit, int stored) {
@@ -592,10 +591,11 @@ static __host__ __device__ inline size_t seed_smem_size(int threads, int smem_hi
            (sizeof(int2) + sizeof(int) + sizeof(uint16_t)) * threads + sizeof(int) * (2 * kScanInts + 16);
 }
 
-static __host__ __device__ inline size_t seed_slot_size(int cand_cap, int max_xhits) {
-    return (sizeof(Cand) + sizeof(int)) * size_t(cand_cap) + sizeof(ull) * (size_t(max_xhits) + cand_cap) + 16 +
-           sizeof(UvRec) * kUvStore + sizeof(float) * 6 * size_t(cand_cap) + 9 * size_t(cand_cap) + 4 +
-           sizeof(uint32_t) * ((size_t(max_xhits) + 31) / 32);
+// max_hits: hits of a half (the taken-hit bits)
+static __host__ __device__ inline size_t seed_slot_size(int cand_cap, int uv_cap, int tbl_cap, int max_hits) {
+    return (sizeof(Cand) + sizeof(int)) * size_t(cand_cap) + sizeof(ull) * (size_t(tbl_cap) + cand_cap) + 16 +
+           sizeof(UvRec) * size_t(uv_cap) + sizeof(float) * 6 * size_t(cand_cap) + 9 * size_t(cand_cap) + 4 +
+           sizeof(uint32_t) * ((size_t(max_hits) + 31) / 32);
 }
 
 constexpr int kDeferRounds = 2;       // matching left to idle CTAs once fewer seeding items than this per CTA remain
@@ -612,8 +612,9 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // A CTA's scratch in global memory (SeedArgs::slot).
 struct SeedSlot {
     int CC;            // candidates an item may have
+    int uv_cap;        // valid UV combinations stored
     Cand* cand;        // [CC] the candidates in the order of the search
-    UvRec* uv;         // [kUvStore] the valid UV combinations
+    UvRec* uv;         // [uv_cap] the valid UV combinations
     ull* tbl;          // clone table, if it does not fit in shared memory
     ull* key;          // UV keys, if they do not
     float* xs;         // x at the stereo layers of the kept seeds, if not in shared memory
@@ -621,12 +622,12 @@ struct SeedSlot {
     uint8_t* hcl;      // Hough variant: kept clusters per seed
     uint8_t* hn;       // and their count
     uint32_t* used;    // HLT2-style mode: bits of the half's hits taken by earlier iterations
-    __device__ __forceinline__ SeedSlot(uint8_t* slot, int cc, int max_xhits) : CC(cc) {
+    __device__ __forceinline__ SeedSlot(uint8_t* slot, int cc, int uvc, int tbl_cap) : CC(cc), uv_cap(uvc) {
         cand = reinterpret_cast<Cand*>(slot);
         uv = reinterpret_cast<UvRec*>(cand + CC);
-        key = reinterpret_cast<ull*>(uv + kUvStore);
+        key = reinterpret_cast<ull*>(uv + uv_cap);
         tbl = key + CC;
-        xs = reinterpret_cast<float*>(tbl + max_xhits);
+        xs = reinterpret_cast<float*>(tbl + tbl_cap);
         kept = reinterpret_cast<int*>(xs + 6 * CC);
         hcl = reinterpret_cast<uint8_t*>(kept + CC);
         hn = hcl + 8 * CC;
@@ -964,7 +965,7 @@ __device__ __forceinline__ void uv_search(const DevParams& P, const SeedItem& it
     const uint32_t* used = kSeq ? S.used : nullptr;
     uint32_t* const list = reinterpret_cast<uint32_t*>(M.phase);
     const int nkp = nk - kb;
-    const int nvs0 = min(V.nvalid, kUvStore);
+    const int nvs0 = min(V.nvalid, S.uv_cap);
     if (tid == 0) V.nlist = 0;
     for (int j = kb + tid; j < nk; j += T) {
         ukey[j] = ~0ull;
@@ -1054,7 +1055,7 @@ __device__ __forceinline__ void uv_search(const DevParams& P, const SeedItem& it
                                       szl[6 + P.uv_init[pass]] + kinit, start_ty(j, pass, kinit), v);
                 if (n >= P.n_uv_min) {
                     const int sidx = atomicAdd(&V.nvalid, 1);
-                    if (sidx < kUvStore) {
+                    if (sidx < S.uv_cap) {
                         S.uv[sidx].v = v;
                         reinterpret_cast<uint2&>(S.uv[sidx].f) = make_uint2(unsigned(j), unsigned(pass) | (unsigned(kinit) << 1));
                     } else {
@@ -1073,7 +1074,7 @@ __device__ __forceinline__ void uv_search(const DevParams& P, const SeedItem& it
         __syncthreads();
     }
     // the stored combinations' fits, one per thread
-    const int nvs = min(V.nvalid, kUvStore);
+    const int nvs = min(V.nvalid, S.uv_cap);
     for (int q = nvs0 + tid; q < nvs; q += T) {
         UvRec* r = S.uv + q;
         const uint2 mt = reinterpret_cast<const uint2&>(r->f);
@@ -1110,7 +1111,7 @@ k_seed(const __grid_constant__ DevParams P, const __grid_constant__ SeedArgs A) 
     __shared__ int sMask[64];
     const int T = blockDim.x, tid = threadIdx.x;
     const SeedSm M(smem, T, A.smem_hits, A.tbl_smem, A.key_smem);
-    const SeedSlot S(A.slot + int64_t(blockIdx.x) * A.slot_stride, A.cand_cap, A.max_xhits);
+    const SeedSlot S(A.slot + int64_t(blockIdx.x) * A.slot_stride, A.cand_cap, A.uv_cap, A.tbl_cap);
     const HitMap map{M.bits, M.first};
     const int* szl = M.szl;
     for (int i = tid; i < kMasks * 18; i += T) sG[kGainRow * (i / 18) + i % 18] = (&P.G[0][0][0])[i];
@@ -1134,7 +1135,7 @@ k_seed(const __grid_constant__ DevParams P, const __grid_constant__ SeedArgs A) 
         __syncthreads();
         if (tid == 0) {
             V.match = -1;
-            const int n2 = static_cast<int>(2 * A.n_events);
+            const int n2 = A.n_list ? *A.n_list : static_cast<int>(2 * A.n_events);
             if (kFuse && fin >= 0 && atomicAdd(A.ev_done + fin, 1) == 1) {
                 // this CTA finished the event's second half (the other half's
                 // records were released before its count; the fence orders
@@ -1299,11 +1300,11 @@ k_seed(const __grid_constant__ DevParams P, const __grid_constant__ SeedArgs A) 
         __syncthreads();
 
         int ncand = 0, nk = 0;
-        bool ok = true;
         const int n_pass = seq ? P.n_iter : 1;
         const int nxh = szl[6];
         const bool tbl_in = nxh <= A.tbl_smem;
-        for (int ipass = 0; ipass < n_pass; ++ipass) {
+        bool ok = tbl_in || nxh <= A.tbl_cap;
+        for (int ipass = 0; ok && ipass < n_pass; ++ipass) {
             const SeedItem I{h, seq ? ipass : 0, seq ? ipass + 1 : P.n_iter, P.uv_mode == 1};
             // ------------------------------------------------------------ XZ
             const int cb0 = ncand, kb = nk;
@@ -1333,7 +1334,7 @@ k_seed(const __grid_constant__ DevParams P, const __grid_constant__ SeedArgs A) 
                 // hit cleanup: this pass's seeds give their hits to no later pass.
                 // Their stereo hits come from the chain store; a pass whose store
                 // overflowed cannot be cleaned up and counts as an overflow.
-                if (V.nvalid > kUvStore) {
+                if (V.nvalid > S.uv_cap) {
                     ok = false;
                     break;
                 }
@@ -1361,10 +1362,14 @@ k_seed(const __grid_constant__ DevParams P, const __grid_constant__ SeedArgs A) 
             V.ctr[3] += ncand;
             V.ctr[6] += V.nvalid;  // every valid UV chain of the item's passes
         }
-        if (!ok || (seq && V.nvalid > kUvStore)) {
+        if (!ok || (seq && V.nvalid > S.uv_cap)) {
             if (tid == 0) {
-                A.status[e] = -3;  // ST_OVERFLOW
-                A.item_count[item] = 0;
+                if (A.retry) {
+                    A.retry[atomicAdd(A.retry_ctr, 1)] = static_cast<int32_t>(item);
+                } else {
+                    A.status[e] = -3;  // ST_OVERFLOW
+                    A.item_count[item] = 0;
+                }
             }
             continue;
         }

@@ -140,7 +140,7 @@ extern "C" int seeding_run_static(const st_config* cfg, const st_hits* H, st_see
     const size_t o_pp = take(sizeof(float) * 8 * size_t(S->cap) + 4);
     const size_t o_ps = take(sizeof(float) * 4 * size_t(S->cap) + 4);
     const size_t o_pn = take(2 * size_t(S->cap) + 4);
-    const size_t slot_stride = up256(seed_slot_bytes(cfg->cand_cap, static_cast<int>(mh)));
+    const size_t slot_stride = up256(seed_slot_bytes(cfg->cand_cap, kUvStore, static_cast<int>(mh), static_cast<int>(mh)));
     const size_t slot_limit =
         std::max(slot_stride, up256(seed_slot_limit_bytes(cfg->cand_cap, static_cast<int>(mh))));
     const size_t fixed = off;
@@ -150,7 +150,19 @@ extern "C" int seeding_run_static(const st_config* cfg, const st_hits* H, st_see
                     "static scratch holds %zu; split the batch or lower seeds cap / cand_cap",
                     fixed + slot_limit, (long long)ne, (long long)mh, (long long)S->cap,
                     size_t(ST_STATIC_SCRATCH_BYTES));
-    const int64_t slots_fit = int64_t((size_t(ST_STATIC_SCRATCH_BYTES) - fixed) / slot_stride);
+    // CTAs with the full scratch per item are few (0.7 MB each by default), so
+    // the items first run with what halves of this size need as a rule, and
+    // those that need more run again after them.  Halves of Run-3-like events
+    // have 0.07 candidates and 0.07 valid UV combinations per hit of the event,
+    // of dense ones (280 tracks) 0.07 and 0.08.  100 Run-3-like events: 495 us
+    // with 17 CTAs at a time, 65 us with one per item.
+    const int64_t room = int64_t(ST_STATIC_SCRATCH_BYTES) - int64_t(fixed);
+    const int64_t slots_fit = room / int64_t(slot_stride);
+    const int small_cands = static_cast<int>(std::min<int64_t>(cfg->cand_cap, 32 + mh / 10));
+    const int small_uv = static_cast<int>(std::min<int64_t>(kUvStore, 32 + mh / 8));
+    const size_t small_stride = up256(seed_slot_bytes(small_cands, small_uv, 0, static_cast<int>(mh)));
+    const int64_t small_fit = room / int64_t(small_stride);
+    const bool two_steps = slots_fit < items && small_fit > slots_fit;
     unsigned char* b = D->base;
 
     // what must start at zero each call: work queues, the pool counter and the
@@ -168,24 +180,27 @@ extern "C" int seeding_run_static(const st_config* cfg, const st_hits* H, st_see
     int bins = 8;
     while (bins < 512 && bins * 96 < mh) bins <<= 1;
     const size_t bsmem = build_smem_bytes(bins, static_cast<int>(mh));
-    const int tbl_smem = cfg->smem_hits / 2, key_smem = std::max(64, cfg->smem_hits / 8);  // as st_create
-    const size_t ssmem = seed_smem_bytes(cfg->threads_seed, cfg->smem_hits, tbl_smem, key_smem);
+    SeedShape shapes[kSeedShapes];
+    const int n_shapes = seed_shapes(*cfg, shapes, true);
     // the shared-memory check of st_create (2 KB left for static shared memory)
     const size_t slimit =
-        std::max(ssmem, seed_smem_limit_bytes(cfg->threads_seed, cfg->smem_hits, tbl_smem, key_smem));
+        std::max(shapes[0].smem, seed_smem_limit_bytes(cfg->threads_seed, cfg->smem_hits, shapes[0].tbl_smem,
+                                                       shapes[0].key_smem));
     if (slimit + 2048 > size_t(D->optin) || bsmem + 2048 > size_t(D->optin))
         return fail(err, err_len, ST_EINVAL,
                     "config needs %zu (seeding) / %zu (containers) bytes of shared memory per CTA; the device "
                     "allows %d", slimit, bsmem, D->optin);
     int bbps = std::max(1, build_blocks_per_sm(cfg->threads_build, bsmem));
-    int sbps = std::max(1, seed_blocks_per_sm(cfg->threads_seed, ssmem));
-    if (cfg->ctas_per_sm > 0) {  // as seeding_run
-        bbps = std::min(bbps, cfg->ctas_per_sm);
-        sbps = std::min(sbps, cfg->ctas_per_sm);
-    }
+    if (cfg->ctas_per_sm > 0) bbps = std::min(bbps, cfg->ctas_per_sm);  // as seeding_run
     const int g_build = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(ne, int64_t(D->n_sms) * bbps)));
-    const int g_seed = static_cast<int>(
-        std::max<int64_t>(1, std::min<int64_t>({items, int64_t(D->n_sms) * sbps, slots_fit})));
+    auto seed_grid = [&](const SeedShape& sh, int64_t fit) {
+        int bps = std::max(1, sh.bps);
+        if (cfg->ctas_per_sm > 0) bps = std::min(bps, cfg->ctas_per_sm);
+        return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>({items, int64_t(D->n_sms) * bps, fit})));
+    };
+    const int64_t fit = two_steps ? small_fit : slots_fit;
+    const SeedShape& sh = pick_seed_shape(shapes, n_shapes, *cfg, items, D->n_sms, fit);
+    const int g_seed = seed_grid(sh, fit);
 
     BuildArgs ba;
     ba.n_events = ne;
@@ -220,14 +235,18 @@ extern "C" int seeding_run_static(const st_config* cfg, const st_hits* H, st_see
     sa.corig = ba.corig;
     sa.zoff = ba.zoff;
     sa.status = S->status;
-    sa.smem_hits = cfg->smem_hits;
-    sa.cand_cap = cfg->cand_cap;
-    sa.tbl_smem = tbl_smem;
-    sa.key_smem = key_smem;
+    auto use_shape = [&](const SeedShape& q) {
+        sa.smem_hits = q.smem_hits;
+        sa.tbl_smem = q.tbl_smem;
+        sa.key_smem = q.key_smem;
+    };
+    use_shape(sh);
+    sa.cand_cap = two_steps ? small_cands : cfg->cand_cap;
+    sa.uv_cap = two_steps ? small_uv : kUvStore;
+    sa.tbl_cap = two_steps ? 0 : static_cast<int32_t>(mh);
     sa.round_hits = cfg->threads_seed;
     sa.slot = b + fixed;
-    sa.slot_stride = static_cast<int64_t>(slot_stride);
-    sa.max_xhits = static_cast<int32_t>(mh);
+    sa.slot_stride = static_cast<int64_t>(two_steps ? small_stride : slot_stride);
     sa.pool_hits = reinterpret_cast<int32_t*>(b + o_ph);
     sa.pool_params = reinterpret_cast<float*>(b + o_pp);
     sa.pool_state = reinterpret_cast<float*>(b + o_ps);
@@ -240,7 +259,23 @@ extern "C" int seeding_run_static(const st_config* cfg, const st_hits* H, st_see
     sa.queue = queues + 1;
     sa.counters = counters;
     sa.fault = queues + 4;  // set if a staging copy was given up on
-    e = launch_seed(P, sa, g_seed, cfg->threads_seed, ssmem, s);
+    if (two_steps) {
+        sa.retry = ba.item_class;  // (not needed any more)
+        sa.retry_ctr = queues + 6;
+    }
+    e = launch_seed(P, sa, g_seed, sh.threads, sh.smem, s);
+    if (e == cudaSuccess && two_steps) {
+        use_shape(shapes[0]);
+        sa.cand_cap = cfg->cand_cap;
+        sa.uv_cap = kUvStore;
+        sa.tbl_cap = static_cast<int32_t>(mh);
+        sa.slot_stride = static_cast<int64_t>(slot_stride);
+        sa.order = sa.retry;
+        sa.n_list = sa.retry_ctr;
+        sa.retry = nullptr;
+        sa.queue = queues + 2;
+        e = launch_seed(P, sa, seed_grid(shapes[0], slots_fit), shapes[0].threads, shapes[0].smem, s);
+    }
     if (e != cudaSuccess) return fail(err, err_len, ST_ECUDA, "k_seed: %s", cudaGetErrorString(e));
 
     GatherArgs ga;

@@ -72,3 +72,28 @@ def test_larger_ctas_give_the_same(mode, zmx):
     for k in KEYS[1:]:
         assert np.array_equal(small[k], big[k][:len(small[k])]), k
     assert n > 0
+
+
+@pytest.mark.parametrize("n,tracks,over", [
+    (60, 150, {}),                                       # one CTA per item
+    (20, 260, {}),                                       # halves with more hits than shared memory holds
+    (48, 60, dict(m_lo=0.0, m_hi=40.0, chi2x_max=1e9)),  # more candidates than the first step's scratch holds
+    (48, 60, dict(uv_tol=40.0, n_uv_min=2)),             # more UV combinations than it holds
+    (48, 60, dict(iter_mode=1, uv_tol=40.0, n_uv_min=2)),
+])
+def test_static_entry_in_two_steps(n, tracks, over, zmx):
+    """seeding_run_static runs the items with little scratch each first and
+    again, with all they may need, those that ask for more."""
+    b = make_events(n, seed=4011, tracks=("fixed", tracks))
+    _, gcfg = parity.config_pair(zmx, **over)
+    ctx = st.Context(gcfg)
+    db = st.DeviceBatch.from_synth(b)
+    cap = max(1024, b.n_hits // 4)
+    ref, out = st.DeviceOutputs(n, cap), st.DeviceOutputs(n, cap)
+    ctx.seeding_run(db.hits, ref.seeds)
+    rc, msg = st.seeding_run_static(gcfg, db.hits, out.seeds)
+    assert rc == st.ST_OK, msg
+    r, g = ref.to_numpy(), out.to_numpy()
+    for k in ("ev_off", "hits", "params", "state", "n_hits", "status"):
+        assert np.array_equal(r[k], g[k]), k
+    ctx.close()
