@@ -9,16 +9,17 @@
 
 namespace st {
 
-// CTAs of the seeding kernel: threads, what their shared memory holds, and how
-// many an SM takes.
+// CTAs of the seeding kernel: threads, whether with more registers each, what
+// their shared memory holds, and how many an SM takes.
 struct SeedShape {
+    bool wide = false;
     int threads = 0, smem_hits = 0, tbl_smem = 0, key_smem = 0, velo_smem = 0;
     size_t smem = 0;
     int bps = 0;
 };
 
-// The shapes a configuration may run with: [0] as configured, then larger CTAs
-// for batches that leave SMs idle.  Returns how many; with `bps`, how many CTAs
+// The shapes a configuration may run with: [0] as configured, then ever fewer
+// CTAs per SM, for smaller batches.  Returns how many; with `bps`, how many CTAs
 // of each an SM takes (after set_smem_limits).
 int seed_shapes(const st_config& c, SeedShape out[kSeedShapes], bool bps);
 

@@ -515,7 +515,7 @@ cudaError_t set_smem_limits(size_t optin) {
     int n = 3;
     for (int sh = 0; sh < kSeedShapes; ++sh)
         for (int mode = 0; mode < 3; ++mode)
-            fns[n++] = reinterpret_cast<const void*>(seed_kernel(kSeedThreads[sh], mode == 1, mode == 2));
+            fns[n++] = reinterpret_cast<const void*>(seed_kernel(kSeedThreads[sh], kSeedWide[sh], mode == 1, mode == 2));
     for (const void* f : fns) {
         cudaFuncAttributes fa;
         cudaError_t err = cudaFuncGetAttributes(&fa, f);
@@ -543,9 +543,9 @@ int build_blocks_per_sm(int threads, size_t smem) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_build, threads, smem);
     return n;
 }
-int seed_blocks_per_sm(int threads, size_t smem) {
+int seed_blocks_per_sm(int threads, bool wide, size_t smem) {
     int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, seed_kernel(threads, false, false), threads, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, seed_kernel(threads, wide, false, false), threads, smem);
     return n;
 }
 int match_blocks_per_sm(int threads, size_t smem, bool final_sel) {
@@ -585,11 +585,11 @@ cudaError_t launch_build(const DevParams& P, const BuildArgs& a, int grid, int t
                     chained, a);
 }
 
-cudaError_t launch_seed(const DevParams& P, const SeedArgs& a, int grid, int threads, size_t smem, cudaStream_t s,
+cudaError_t launch_seed(const DevParams& P, const SeedArgs& a, int grid, int threads, bool wide, size_t smem, cudaStream_t s,
                         bool chained) {
     const bool sq = P.iter_mode == 1;
     if (a.velo && sq) return cudaErrorInvalidValue;  // the runtime asks for fused matching in the HLT1 mode only
-    const SeedKernel k = seed_kernel(threads, sq, a.velo != nullptr);
+    const SeedKernel k = seed_kernel(threads, wide, sq, a.velo != nullptr);
     return launch_k(k, static_cast<unsigned>(grid), static_cast<unsigned>(threads), smem, s, chained, P, a);
 }
 

@@ -130,14 +130,16 @@ struct MatchArgs {
     unsigned long long* counters;
 };
 
-// The seeding kernel comes in CTAs of up to kSeedThreads[i] threads; its
-// instantiations are spread over translation units that compile in parallel.
-constexpr int kSeedShapes = 3;
-constexpr int kSeedThreads[kSeedShapes] = {256, 448, 512};
+// The seeding kernel comes in CTAs of up to kSeedThreads[i] threads, those of
+// 256 with fewer registers per thread or (wide) more; its instantiations are
+// spread over translation units that compile in parallel.
+constexpr int kSeedShapes = 4;
+constexpr int kSeedThreads[kSeedShapes] = {256, 256, 384, 512};
+constexpr bool kSeedWide[kSeedShapes] = {false, true, false, false};
 typedef void (*SeedKernel)(const DevParams, const SeedArgs);
 // the instantiation for CTAs of `threads` threads, with the HLT2-style pass
 // loop (seq) or with the matching fused in
-SeedKernel seed_kernel(int threads, bool seq, bool fused);
+SeedKernel seed_kernel(int threads, bool wide, bool seq, bool fused);
 
 size_t build_smem_bytes(int bins, int smem_hits);
 size_t seed_smem_bytes(int threads, int smem_hits, int tbl_smem, int key_smem);
@@ -154,14 +156,14 @@ size_t match_smem_bytes(int velo_smem);
 // stream's kernels want those SMs.
 cudaError_t launch_build(const DevParams& P, const BuildArgs& a, int grid, int threads, cudaStream_t s,
                          bool chained = true);
-cudaError_t launch_seed(const DevParams& P, const SeedArgs& a, int grid, int threads, size_t smem, cudaStream_t s,
+cudaError_t launch_seed(const DevParams& P, const SeedArgs& a, int grid, int threads, bool wide, size_t smem, cudaStream_t s,
                         bool chained = true);
 cudaError_t launch_gather(const GatherArgs& a, cudaStream_t s, bool chained = true);
 cudaError_t launch_match(const DevParams& P, const MatchArgs& a, int grid, int threads, cudaStream_t s);
 
 // occupancy helpers
 int build_blocks_per_sm(int threads, size_t smem);
-int seed_blocks_per_sm(int threads, size_t smem);
+int seed_blocks_per_sm(int threads, bool wide, size_t smem);
 int match_blocks_per_sm(int threads, size_t smem, bool final_sel);
 cudaError_t set_smem_limits(size_t optin);
 cudaError_t smem_limits_hold(size_t optin, bool& hold);

@@ -388,34 +388,43 @@ namespace st {
 
 int seed_shapes(const st_config& c, SeedShape out[kSeedShapes], bool bps) {
     int n = 0;
-    auto add = [&](int threads, int smem_hits, int velo_smem) {
+    auto add = [&](int threads, bool wide, int smem_hits, int velo_smem) {
         SeedShape& s = out[n++];
         s.threads = threads;
+        s.wide = wide;
         s.smem_hits = smem_hits;
         s.tbl_smem = smem_hits / 2;
         s.key_smem = std::max(64, smem_hits / 8);  // kept seeds whose UV keys and stereo x stay in shared memory
         s.velo_smem = velo_smem;
         s.smem = std::max(seed_smem_bytes(threads, smem_hits, s.tbl_smem, s.key_smem), match_smem_bytes(velo_smem));
-        s.bps = bps ? seed_blocks_per_sm(threads, s.smem) : 0;
+        s.bps = bps ? seed_blocks_per_sm(threads, wide, s.smem) : 0;
     };
-    add(c.threads_seed, c.smem_hits, 512);
-    if (c.threads_seed < 448) add(448, 2048, 768);
-    if (c.threads_seed < 512) add(512, 4096, 1024);
+    add(c.threads_seed, false, c.smem_hits, 512);
+    if (c.threads_seed <= 256) add(256, true, std::max(c.smem_hits, 1536), 512);
+    if (c.threads_seed < 384) add(384, false, 2048, 768);
+    if (c.threads_seed < 512) add(512, false, 4096, 1024);
     return n;
 }
 
 // The largest CTAs that take the batch in one round.  Such a batch is bound by
 // the latency of one item, which falls with the threads that share it; above
 // that the SMs are shared anyway and the smaller CTAs pass their barriers
-// sooner.  k_seed, Run-3-like events, at 256 / 448 / 512 threads: 67 events 69 /
-// 57 / 53 us, 150 events 90 / 71 / 65, 220 events 91 / 81 / 85, 300 events 91 /
-// 96 / 95, 1000 events 191 / 233 / 271.  A set ctas_per_sm asks for the
-// configured shape.
+// sooner.  Of the CTAs of 256 threads, four to an SM with 64 registers a thread
+// spill less (450 bytes against 860) than five with 48, which pays until five
+// hide each other's latency over several rounds.  k_seed, Run-3-like events, at
+// 256 / 448 / 512 threads: 67 events 69 / 57 / 53 us, 150 events 90 / 71 / 65,
+// 220 events 91 / 81 / 85.  The whole step at 448 / 384 threads: 200 events 98 /
+// 95 us, 225 events 96 / 94; at 256 threads five / four to an SM: 250 events
+// 113 / 109, 300 events 122 / 114, 450 events 139 / 136, 600 events 160 / 154,
+// 900 events 217 / 213, 1000 events 232 / 237, 2000 events 444 / 452.  A set
+// ctas_per_sm asks for the configured shape.
 const SeedShape& pick_seed_shape(const SeedShape* shapes, int n, const st_config& c, int64_t items, int n_sms,
                                  int64_t max_ctas) {
     if (c.ctas_per_sm == 0)
-        for (int k = n - 1; k > 0; --k)
-            if (items <= std::min<int64_t>(int64_t(n_sms) * shapes[k].bps, max_ctas)) return shapes[k];
+        for (int k = n - 1; k > 0; --k) {
+            const int64_t ctas = std::min<int64_t>(int64_t(n_sms) * shapes[k].bps, max_ctas);
+            if (items <= (shapes[k].wide ? ctas * 5 / 2 : ctas)) return shapes[k];
+        }
     return shapes[0];
 }
 
@@ -818,7 +827,7 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
         if (ctx->timing && &w == &ctx->ws) ctx->tused[3] = false;  // matching runs inside k_seed
     }
     tmark(ctx, w, 1, 0, s);
-    ST_CUDA(ctx, launch_seed(ctx->P, a, g_seed, sh.threads, sh.smem, s, chain && !marks));
+    ST_CUDA(ctx, launch_seed(ctx->P, a, g_seed, sh.threads, sh.wide, sh.smem, s, chain && !marks));
     tmark(ctx, w, 1, 1, s);
 
     GatherArgs g;

@@ -25,9 +25,9 @@ size_t seed_slot_limit_bytes(int cand_cap, int max_xhits) {
            sizeof(ull) * 12 * 512 + 9 * size_t(cand_cap) + 4 + sizeof(uint32_t) * ((size_t(max_xhits) + 31) / 32);
 }
 
-SeedKernel seed_kernel(int threads, bool seq, bool fused) {
-    return threads <= 256 ? seed_kernel_256(seq, fused)
-           : threads <= 448 ? seed_kernel_448(seq, fused)
+SeedKernel seed_kernel(int threads, bool wide, bool seq, bool fused) {
+    return threads <= 256 ? (wide ? seed_kernel_256w(seq, fused) : seed_kernel_256(seq, fused))
+           : threads <= 384 ? seed_kernel_384(seq, fused)
                             : seed_kernel_512(seq, fused);
 }
 

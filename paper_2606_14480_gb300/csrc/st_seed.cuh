@@ -23,12 +23,14 @@
 
 namespace st {
 
-// CTAs per SM of each shape (48 registers per thread, 64 for the last)
+// CTAs per SM of each shape: 48, 64, 56 and 64 registers per thread
 constexpr int kSeedBlocks256 = 5;
-constexpr int kSeedBlocks448 = 3;
+constexpr int kSeedBlocks256w = 4;
+constexpr int kSeedBlocks384 = 3;
 constexpr int kSeedBlocks512 = 2;
 SeedKernel seed_kernel_256(bool seq, bool fused);
-SeedKernel seed_kernel_448(bool seq, bool fused);
+SeedKernel seed_kernel_256w(bool seq, bool fused);
+SeedKernel seed_kernel_384(bool seq, bool fused);
 SeedKernel seed_kernel_512(bool seq, bool fused);
 
 // ---------------------------------------------------------------------------

@@ -263,7 +263,7 @@ extern "C" int seeding_run_static(const st_config* cfg, const st_hits* H, st_see
         sa.retry = ba.item_class;  // (not needed any more)
         sa.retry_ctr = queues + 6;
     }
-    e = launch_seed(P, sa, g_seed, sh.threads, sh.smem, s);
+    e = launch_seed(P, sa, g_seed, sh.threads, sh.wide, sh.smem, s);
     if (e == cudaSuccess && two_steps) {
         use_shape(shapes[0]);
         sa.cand_cap = cfg->cand_cap;
@@ -274,7 +274,7 @@ extern "C" int seeding_run_static(const st_config* cfg, const st_hits* H, st_see
         sa.n_list = sa.retry_ctr;
         sa.retry = nullptr;
         sa.queue = queues + 2;
-        e = launch_seed(P, sa, seed_grid(shapes[0], slots_fit), shapes[0].threads, shapes[0].smem, s);
+        e = launch_seed(P, sa, seed_grid(shapes[0], slots_fit), shapes[0].threads, shapes[0].wide, shapes[0].smem, s);
     }
     if (e != cudaSuccess) return fail(err, err_len, ST_ECUDA, "k_seed: %s", cudaGetErrorString(e));
 

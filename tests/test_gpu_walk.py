@@ -2,7 +2,7 @@
 
 Pairs are walked in groups of 32 and blocks of 12 groups per warp, triplets
 wait in queues of 128 per warp, UV combinations go in blocks of 1024, and
-batches of up to two items per SM run in larger CTAs.  Wide third-hit bands and
+batches of up to ten items per SM run in larger CTAs or with more registers.  Wide third-hit bands and
 windows, tiny events and batch sizes around that limit reach every branch; the
 oracle, and the same batch in CTAs of other sizes, say what is right."""
 
@@ -59,11 +59,12 @@ def test_walk_edges_parity_and_shapes(n, tracks, over, zmx):
             assert np.array_equal(other[k], gpu[k]), (shape, k)
 
 
+@pytest.mark.parametrize("items", [2, 3, 4, 10])
 @pytest.mark.parametrize("mode", [{}, dict(uv_mode=1), dict(iter_mode=1)], ids=["hlt1", "hough", "seq"])
-def test_larger_ctas_give_the_same(mode, zmx):
-    """Around the largest batch that the larger CTAs take in one round: every
-    event's result is that of the batch one event larger."""
-    sms = torch.cuda.get_device_properties(0).multi_processor_count
+def test_larger_ctas_give_the_same(mode, items, zmx):
+    """Around the largest batch (items per SM) that each kind of larger CTAs
+    takes: every event's result is that of the batch one event larger."""
+    sms = items * torch.cuda.get_device_properties(0).multi_processor_count // 2
     b = workload("run3", n_events=sms + 1)
     big = run(b, zmx, **mode)
     small = run(b.subset(range(sms)), zmx, **mode)
