@@ -410,20 +410,22 @@ int seed_shapes(const st_config& c, SeedShape out[kSeedShapes], bool bps) {
 // the latency of one item, which falls with the threads that share it; above
 // that the SMs are shared anyway and the smaller CTAs pass their barriers
 // sooner.  Of the CTAs of 256 threads, four to an SM with 64 registers a thread
-// spill less (450 bytes against 860) than five with 48, which pays until five
-// hide each other's latency over several rounds.  k_seed, Run-3-like events, at
+// spill less (570 bytes against 840) than five with 48, which pays for up to two
+// rounds where they are as many as five to an SM need.  k_seed, Run-3-like events, at
 // 256 / 448 / 512 threads: 67 events 69 / 57 / 53 us, 150 events 90 / 71 / 65,
 // 220 events 91 / 81 / 85.  The whole step at 448 / 384 threads: 200 events 98 /
 // 95 us, 225 events 96 / 94; at 256 threads five / four to an SM: 250 events
-// 113 / 109, 300 events 122 / 114, 450 events 139 / 136, 600 events 160 / 154,
-// 900 events 217 / 213, 1000 events 232 / 237, 2000 events 444 / 452.  A set
-// ctas_per_sm asks for the configured shape.
+// 106 / 104, 300 events 112 / 109, 350 events 114 / 118, 450 events 131 / 130,
+// 600 events 151 / 146, 760 events 176 / 182, 900 events 202 / 202, 1000 events
+// 215 / 224, 2000 events 403 / 421.  A set ctas_per_sm asks for the configured
+// shape.
 const SeedShape& pick_seed_shape(const SeedShape* shapes, int n, const st_config& c, int64_t items, int n_sms,
                                  int64_t max_ctas) {
+    auto ctas = [&](int k) { return std::min<int64_t>(int64_t(n_sms) * shapes[k].bps, max_ctas); };
     if (c.ctas_per_sm == 0)
         for (int k = n - 1; k > 0; --k) {
-            const int64_t ctas = std::min<int64_t>(int64_t(n_sms) * shapes[k].bps, max_ctas);
-            if (items <= (shapes[k].wide ? ctas * 5 / 2 : ctas)) return shapes[k];
+            if (items <= ctas(k)) return shapes[k];
+            if (shapes[k].wide && items > ctas(0) && items <= 2 * ctas(k)) return shapes[k];
         }
     return shapes[0];
 }

@@ -23,11 +23,15 @@
 
 namespace st {
 
-// CTAs per SM of each shape: 48, 64, 56 and 64 registers per thread
-constexpr int kSeedBlocks256 = 5;
-constexpr int kSeedBlocks256w = 4;
-constexpr int kSeedBlocks384 = 3;
-constexpr int kSeedBlocks512 = 2;
+// Registers per thread of each shape, for five, four, three and two CTAs per
+// SM.  Set outright: asked for as a number of CTAs per SM (launch bounds), the
+// same counts gave code that was slower everywhere (1000 Run-3-like events 232
+// against 215 us, 301 by direct calls 107 against 101, HLT2-style 250 events
+// 137 against 129).
+constexpr int kSeedRegs256 = 48;
+constexpr int kSeedRegs256w = 64;
+constexpr int kSeedRegs384 = 56;
+constexpr int kSeedRegs512 = 64;
 SeedKernel seed_kernel_256(bool seq, bool fused);
 SeedKernel seed_kernel_256w(bool seq, bool fused);
 SeedKernel seed_kernel_384(bool seq, bool fused);
@@ -1102,8 +1106,8 @@ __device__ __forceinline__ void uv_search(const DevParams& P, const SeedItem& it
 // some event is still being seeded by a running CTA.  Kernels that share the
 // GPU with others (the serving pipeline) do not defer: a waiting CTA would
 // hold resources the other kernels could use.
-template <int kT, int kB, bool kSeq, bool kFuse>
-__global__ void __launch_bounds__(kT, kB)
+template <int kT, int kR, bool kSeq, bool kFuse>
+__global__ void __launch_bounds__(kT) __maxnreg__(kR)
 k_seed(const __grid_constant__ DevParams P, const __grid_constant__ SeedArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ SeedVars V;
@@ -1472,9 +1476,9 @@ k_seed(const __grid_constant__ DevParams P, const __grid_constant__ SeedArgs A) 
     if (kFuse && tid == 3 && V.mctr[3]) atomicAdd(A.counters + C_MATCH_EVAL, V.mctr[3]);
 }
 
-template <int kT, int kB>
+template <int kT, int kR>
 SeedKernel seed_kernel_of(bool seq, bool fused) {
-    return fused ? k_seed<kT, kB, false, true> : seq ? k_seed<kT, kB, true, false> : k_seed<kT, kB, false, false>;
+    return fused ? k_seed<kT, kR, false, true> : seq ? k_seed<kT, kR, true, false> : k_seed<kT, kR, false, false>;
 }
 
 }  // namespace st

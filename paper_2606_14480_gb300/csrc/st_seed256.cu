@@ -3,6 +3,6 @@
 
 namespace st {
 
-SeedKernel seed_kernel_256(bool seq, bool fused) { return seed_kernel_of<256, kSeedBlocks256>(seq, fused); }
+SeedKernel seed_kernel_256(bool seq, bool fused) { return seed_kernel_of<256, kSeedRegs256>(seq, fused); }
 
 }  // namespace st

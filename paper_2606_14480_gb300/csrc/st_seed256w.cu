@@ -4,6 +4,6 @@
 
 namespace st {
 
-SeedKernel seed_kernel_256w(bool seq, bool fused) { return seed_kernel_of<256, kSeedBlocks256w>(seq, fused); }
+SeedKernel seed_kernel_256w(bool seq, bool fused) { return seed_kernel_of<256, kSeedRegs256w>(seq, fused); }
 
 }  // namespace st

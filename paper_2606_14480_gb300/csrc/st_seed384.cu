@@ -3,6 +3,6 @@
 
 namespace st {
 
-SeedKernel seed_kernel_384(bool seq, bool fused) { return seed_kernel_of<384, kSeedBlocks384>(seq, fused); }
+SeedKernel seed_kernel_384(bool seq, bool fused) { return seed_kernel_of<384, kSeedRegs384>(seq, fused); }
 
 }  // namespace st

@@ -3,6 +3,6 @@
 
 namespace st {
 
-SeedKernel seed_kernel_512(bool seq, bool fused) { return seed_kernel_of<512, kSeedBlocks512>(seq, fused); }
+SeedKernel seed_kernel_512(bool seq, bool fused) { return seed_kernel_of<512, kSeedRegs512>(seq, fused); }
 
 }  // namespace st
