@@ -1231,10 +1231,6 @@ k_seed(const __grid_constant__ DevParams P, const __grid_constant__ SeedArgs A) 
         const int64_t e = item >> 1;
         const int h = static_cast<int>(item & 1);
         if (kFuse) fin = e;
-        if (A.status[e] != 0) {
-            if (tid == 0) A.item_count[item] = 0;
-            continue;
-        }
         const int32_t* zo = A.zoff + e * kZoffStride + 12 * h;
         const int64_t cbh = cont_base(A.ev_off, e) + zo[0];
         const int nh = zo[12] - zo[0];
