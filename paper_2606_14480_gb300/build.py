@@ -18,7 +18,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libst.so")
-SOURCES = ("st_seed256.cu", "st_seed256w.cu", "st_seed384.cu", "st_seed512.cu", "st_seed.cu", "st_kernels.cu",
+SOURCES = ("st_seed256.cu", "st_seed256w.cu", "st_seed384.cu", "st_seed512.cu", "st_seed1024.cu", "st_seed.cu", "st_kernels.cu",
            "st_runtime.cu", "st_static.cu", "st_ut.cu")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -89,14 +89,20 @@ size_t build_smem_bytes(int bins, int smem_hits) {
 // counts are cleared during the ranking and the next event's ticket and
 // offsets are fetched during the placement, so the next event starts with
 // its loads.  At most 32 registers: up to eight 256-thread CTAs per SM.
-__global__ void __launch_bounds__(kMaxThreads, 4)
+//
+// A batch that may hold large events is shared by two launches side by side
+// (BuildArgs::split_hits): kLarge takes the events above it in CTAs with most
+// of an SM's shared memory (an event of 12,700 hits: 82 us in scratch memory
+// before), the other the rest with little of it each.
+template <bool kLarge>
+__global__ void __launch_bounds__(kMaxThreads, kLarge ? 1 : 4)
 k_build(const __grid_constant__ DevParams P, const __grid_constant__ BuildArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int B = A.bins, NB = kZones * B, T = blockDim.x, tid = threadIdx.x;
+    const int NBmax = kZones * A.bins, T = blockDim.x, tid = threadIdx.x;
     int* cnt = reinterpret_cast<int*>(smem);  // counts, then fill cursors, then cleared
-    int* off = cnt + NB;
-    int* tmp = off + NB + 1;
-    unsigned char* harea = smem + align16(sizeof(int) * (2 * NB + 1 + kScanInts));
+    int* off = cnt + NBmax;
+    int* tmp = off + NBmax + 1;
+    unsigned char* harea = smem + align16(sizeof(int) * (2 * NBmax + 1 + kScanInts));
     // the CTA's next event and its hit range, published by thread 0
     __shared__ int s_item, s_bad;
     __shared__ long long s_h0, s_h1;
@@ -111,24 +117,56 @@ k_build(const __grid_constant__ DevParams P, const __grid_constant__ BuildArgs A
     }
     ull ctr[2] = {0, 0};
     int spar = 0;  // which half of tmp the next block scan uses
-    for (int k = tid; k < NB; k += T) cnt[k] = 0;
+    for (int k = tid; k < NBmax; k += T) cnt[k] = 0;
+    // the first warp: the next event and its offsets.  Tickets, or the next
+    // large one of every gridDim.x-th event, 32 of them looked at together.
+    __shared__ long long s_scan;
+    auto next_item = [&]() {
+        if constexpr (kLarge) {
+            int64_t e = A.n_events;
+            int64_t h0 = 0, h1 = 0;
+            int64_t k = s_scan;
+            for (; k < A.n_events; k += 32 * int64_t(gridDim.x)) {
+                const int64_t c = k + tid * int64_t(gridDim.x);
+                if (c < A.n_events) {
+                    h0 = A.ev_off[c];
+                    h1 = A.ev_off[c + 1];
+                }
+                const unsigned hit =
+                    __ballot_sync(0xffffffffu, c < A.n_events && h1 - h0 > A.split_hits && h1 - h0 <= A.max_hits);
+                if (hit) {
+                    const int l = __ffs(hit) - 1;
+                    e = k + l * int64_t(gridDim.x);
+                    if (tid == l) {
+                        s_h0 = h0;
+                        s_h1 = h1;
+                    }
+                    break;
+                }
+            }
+            __syncwarp();
+            if (tid == 0) {
+                s_scan = e + gridDim.x;
+                s_item = static_cast<int>(e);
+            }
+            __syncwarp();
+        } else if (tid == 0) {
+            const int q = atomicAdd(A.queue, 1);
+            if (q < A.n_events) {
+                s_h0 = A.ev_off[q];
+                s_h1 = A.ev_off[q + 1];
+            }
+            s_item = q;
+        }
+    };
     if (tid == 0) {
         s_bad = 0;
-        s_item = atomicAdd(A.queue, 1);
-        if (s_item < A.n_events) {
-            s_h0 = A.ev_off[s_item];
-            s_h1 = A.ev_off[s_item + 1];
-        }
+        s_scan = blockIdx.x;
     }
-    // thread 0: the next ticket and the offsets of its event
-    auto next_item = [&]() {
-        const int q = atomicAdd(A.queue, 1);
-        if (q < A.n_events) {
-            s_h0 = A.ev_off[q];
-            s_h1 = A.ev_off[q + 1];
-        }
-        s_item = q;
-    };
+    if (tid < 32) {
+        __syncwarp();
+        next_item();
+    }
 
     for (;;) {
         __syncthreads();
@@ -138,19 +176,27 @@ k_build(const __grid_constant__ DevParams P, const __grid_constant__ BuildArgs A
         const int64_t n64 = s_h1 - h0;
         int32_t* zo = A.zoff + e * kZoffStride;
         const int64_t cb = cont_base(A.ev_off, e);
-        if (n64 < 0 || n64 > A.max_hits || cb + n64 > A.cont_cap) {
+        const bool bad_size = n64 < 0 || n64 > A.max_hits || cb + n64 > A.cont_cap;
+        if (kLarge ? bad_size : !bad_size && A.split_hits > 0 && n64 > A.split_hits) {
+            __syncthreads();  // the other launch's
+            if (tid < 32) next_item();
+            continue;
+        }
+        if (bad_size) {
             // too large for max_hits, or an earlier oversized event pushed this
             // one past the container
             for (int k = tid; k < kZoffStride; k += T) zo[k] = 0;
             if (tid < 2) set_item_class(A, 2 * e + tid, 0);
             __syncthreads();  // every thread has read s_item
-            if (tid == 0) {
-                A.status[e] = -3;  // ST_OVERFLOW
-                next_item();
-            }
+            if (tid == 0) A.status[e] = -3;  // ST_OVERFLOW
+            if (tid < 32) next_item();
             continue;
         }
         const int n = static_cast<int>(n64);
+        // about four hits per bucket
+        int B = min(8, A.bins);
+        while (B < A.bins && B * (4 * kZones) < n) B <<= 1;
+        const int NB = kZones * B;
         const bool in_smem = n <= A.smem_hits;
         unsigned char* base = in_smem ? harea : A.big + int64_t(blockIdx.x) * A.big_stride;
         const int cap = in_smem ? A.smem_hits : A.max_hits;
@@ -202,8 +248,8 @@ k_build(const __grid_constant__ DevParams P, const __grid_constant__ BuildArgs A
             if (tid == 0) {
                 A.status[e] = -1;  // ST_EINVAL
                 s_bad = 0;
-                next_item();
             }
+            if (tid < 32) next_item();
             continue;
         }
         {   // exclusive scan of the bucket counts; the counts become fill cursors
@@ -222,7 +268,7 @@ k_build(const __grid_constant__ DevParams P, const __grid_constant__ BuildArgs A
             if (tid == 0) off[NB] = tot;
         }
         __syncthreads();
-        if (tid == 0) next_item();  // read by the other threads after the next loop-top barrier
+        if (tid < 32) next_item();  // read by the other threads after the next loop-top barrier
         for (int i = tid; i < n; i += T) pm[atomicAdd(&cnt[bk[i]], 1)] = static_cast<uint16_t>(i);
         __syncthreads();
         // rank of each hit in its bucket -> its place in the sorted event;
@@ -276,6 +322,10 @@ k_build(const __grid_constant__ DevParams P, const __grid_constant__ BuildArgs A
 // The order inside a class does not matter: items are independent and their
 // results are gathered per event.
 constexpr int kOrderThreads = 1024;
+// The items for the larger CTAs of a split batch: those that cost this many
+// times the mean.  2000 uneven events (120 tracks on average) / 500 of them, at
+// 4, 5, 6.5 times: 698 / 483, 679 / 492, 664 / 503 us.
+constexpr float kBigCost = 5.f;
 
 __global__ void __launch_bounds__(kOrderThreads) k_order(const __grid_constant__ BuildArgs A) {
     __shared__ int pos[kCostClasses], s_cnt[kCostClasses];
@@ -307,6 +357,20 @@ __global__ void __launch_bounds__(kOrderThreads) k_order(const __grid_constant__
     for (int k = tid; k < kCostClasses; k += kOrderThreads) s_cnt[k] = 0;
     __syncthreads();
     const int64_t items = 2 * A.n_events;
+    if (A.n_big && blockIdx.x == 0 && tid < 32) {
+        auto cost = [](int c) {  // the least cost of class c (cost_class)
+            return c < 8 ? float(c) : ldexpf(float(4 + (c & 3)), (c >> 2) - 2);
+        };
+        float sum = 0.f;
+        for (int c = tid; c < kCostClasses; c += 32) sum += cost(c) * float(A.class_count[c]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        const float bar = kBigCost * sum / float(items);
+        int n = 0;
+        for (int c = tid; c < kCostClasses; c += 32) n += cost(c) >= bar ? A.class_count[c] : 0;
+        n = __reduce_add_sync(0xffffffffu, n);
+        if (tid == 0) *A.n_big = n;
+    }
     const int64_t i = int64_t(blockIdx.x) * kOrderThreads + tid;
     const int c = i < items ? A.item_class[i] : -1;
     const unsigned same = __match_any_sync(0xffffffffu, c);
@@ -509,10 +573,11 @@ size_t match_smem_bytes(int velo_smem) { return match_smem_size(velo_smem); }
 // Raise each kernel's dynamic shared-memory ceiling to what the device allows
 // next to the kernel's own static shared memory (opt-in maximum - static).
 cudaError_t set_smem_limits(size_t optin) {
-    const void* fns[3 + 3 * kSeedShapes] = {reinterpret_cast<const void*>(k_build),
+    const void* fns[4 + 3 * kSeedShapes] = {reinterpret_cast<const void*>(k_build<false>),
+                                            reinterpret_cast<const void*>(k_build<true>),
                                             reinterpret_cast<const void*>(k_match<false>),
                                             reinterpret_cast<const void*>(k_match<true>)};
-    int n = 3;
+    int n = 4;
     for (int sh = 0; sh < kSeedShapes; ++sh)
         for (int mode = 0; mode < 3; ++mode)
             fns[n++] = reinterpret_cast<const void*>(seed_kernel(kSeedThreads[sh], kSeedWide[sh], mode == 1, mode == 2));
@@ -532,7 +597,7 @@ cudaError_t set_smem_limits(size_t optin) {
 // kernel, the first one set_smem_limits raises.
 cudaError_t smem_limits_hold(size_t optin, bool& hold) {
     cudaFuncAttributes fa;
-    const cudaError_t err = cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(k_build));
+    const cudaError_t err = cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(k_build<false>));
     hold = err == cudaSuccess &&
            fa.maxDynamicSharedSizeBytes >= static_cast<int>(optin) - static_cast<int>(fa.sharedSizeBytes);
     return err;
@@ -540,7 +605,7 @@ cudaError_t smem_limits_hold(size_t optin, bool& hold) {
 
 int build_blocks_per_sm(int threads, size_t smem) {
     int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_build, threads, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_build<false>, threads, smem);
     return n;
 }
 int seed_blocks_per_sm(int threads, bool wide, size_t smem) {
@@ -558,39 +623,53 @@ int match_blocks_per_sm(int threads, size_t smem, bool final_sel) {
 }
 
 // A launch as a programmatic dependent of the stream's previous kernel
-// (chained), or a plain one.
+// (chained), or a plain one; `started` (if given) is recorded when all its
+// CTAs have begun.
 template <typename... KArgs, typename... Args>
 static cudaError_t launch_k(void (*k)(KArgs...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s,
-                            bool chained, Args&&... args) {
+                            bool chained, cudaEvent_t started, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute at[2];
     cfg.attrs = at;
-    cfg.numAttrs = chained ? 1 : 0;
+    if (chained) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (started) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeLaunchCompletionEvent;
+        at[cfg.numAttrs].val.launchCompletionEvent.event = started;
+        at[cfg.numAttrs++].val.launchCompletionEvent.flags = 0;
+    }
     return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
 }
 
-cudaError_t launch_build(const DevParams& P, const BuildArgs& a, int grid, int threads, cudaStream_t s, bool chained) {
-    k_build<<<grid, threads, build_smem_bytes(a.bins, a.smem_hits), s>>>(P, a);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+cudaError_t launch_build(const DevParams& P, const BuildArgs& a, int grid, int threads, cudaStream_t s) {
+    return launch_k(k_build<false>, static_cast<unsigned>(grid), static_cast<unsigned>(threads),
+                    build_smem_bytes(a.bins, a.smem_hits), s, false, nullptr, P, a);
+}
+
+cudaError_t launch_build_large(const DevParams& P, const BuildArgs& a, int grid, cudaStream_t s, cudaEvent_t started) {
+    return launch_k(k_build<true>, static_cast<unsigned>(grid), kMaxThreads, build_smem_bytes(a.bins, a.smem_hits), s,
+                    false, started, P, a);
+}
+
+cudaError_t launch_order(const BuildArgs& a, cudaStream_t s, bool chained) {
     const int64_t items = 2 * a.n_events;
     if (items <= 0 || !a.order) return cudaSuccess;
     return launch_k(k_order, static_cast<unsigned>((items + kOrderThreads - 1) / kOrderThreads), kOrderThreads, 0, s,
-                    chained, a);
+                    chained, nullptr, a);
 }
 
-cudaError_t launch_seed(const DevParams& P, const SeedArgs& a, int grid, int threads, bool wide, size_t smem, cudaStream_t s,
-                        bool chained) {
+cudaError_t launch_seed(const DevParams& P, const SeedArgs& a, int grid, int threads, bool wide, size_t smem,
+                        cudaStream_t s, bool chained, cudaEvent_t started) {
     const bool sq = P.iter_mode == 1;
     if (a.velo && sq) return cudaErrorInvalidValue;  // the runtime asks for fused matching in the HLT1 mode only
     const SeedKernel k = seed_kernel(threads, wide, sq, a.velo != nullptr);
-    return launch_k(k, static_cast<unsigned>(grid), static_cast<unsigned>(threads), smem, s, chained, P, a);
+    return launch_k(k, static_cast<unsigned>(grid), static_cast<unsigned>(threads), smem, s, chained, started, P, a);
 }
 
 cudaError_t launch_gather(const GatherArgs& a, cudaStream_t s, bool chained) {
@@ -598,7 +677,7 @@ cudaError_t launch_gather(const GatherArgs& a, cudaStream_t s, bool chained) {
     // short against a kernel of their own
     const bool own = a.n_events <= 2048;
     if (!own) {
-        cudaError_t err = launch_k(k_scan, 1, 1024, 0, s, chained, a);
+        cudaError_t err = launch_k(k_scan, 1, 1024, 0, s, chained, nullptr, a);
         if (err != cudaSuccess) return err;
     }
     const int grid = static_cast<int>(std::min<int64_t>(a.n_events, 8192));
@@ -609,7 +688,7 @@ cudaError_t launch_gather(const GatherArgs& a, cudaStream_t s, bool chained) {
     const bool vec = mis == 0 && (reinterpret_cast<uintptr_t>(a.n_hits) & 1u) == 0;
     void (*k)(const GatherArgs) = own ? (vec ? k_gather<true, true> : k_gather<false, true>)
                                       : (vec ? k_gather<true, false> : k_gather<false, false>);
-    return launch_k(k, static_cast<unsigned>(grid), 256, 0, s, own ? chained : true, a);
+    return launch_k(k, static_cast<unsigned>(grid), 256, 0, s, own ? chained : true, nullptr, a);
 }
 
 cudaError_t launch_match(const DevParams& P, const MatchArgs& a, int grid, int threads, cudaStream_t s) {

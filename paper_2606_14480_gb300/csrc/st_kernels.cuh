@@ -22,8 +22,9 @@ struct BuildArgs {
     const float* z;       // may be null
     const float* dxdy;    // may be null
     int32_t max_hits;
-    int32_t bins;         // buckets per container slot (power of two)
+    int32_t bins;         // most buckets per container slot (power of two)
     int32_t smem_hits;    // per-hit arrays in shared memory up to this many hits
+    int32_t split_hits = 0;  // two launches share the events: above this many hits, and the others; 0: one launch
     int64_t cont_cap;     // entries of cx / corig
     float* cx;            // container x
     int32_t* corig;       // container: event-local hit index
@@ -35,6 +36,7 @@ struct BuildArgs {
     int32_t* class_count; // [128] items per class, zero before the launch
     int32_t* class_fill;  // [128] places taken per class, zero before the launch
     int32_t* order;       // [2 n_events] the seeding items, costliest class first; null: not needed
+    int32_t* n_big = nullptr;  // (k_order) out: the items at the front of `order` that cost kBigCost times the mean
     int32_t* queue;
     unsigned long long* counters;
 };
@@ -66,6 +68,9 @@ struct SeedArgs {
     int32_t* item_count;
     const int32_t* order;  // the order of the items; null: each CTA has the one item of its own number
     const int32_t* n_list = nullptr;  // on the device: items in `order`; null: 2 n_events
+    // two launches share `order`: its first *n_big items (part 1) and the others (part 2); part 0: one launch
+    int32_t part = 0;
+    const int32_t* n_big = nullptr;
     // items that need more scratch than a CTA has are listed here for a launch
     // with more; null: their events get ST_OVERFLOW
     int32_t* retry = nullptr;
@@ -133,9 +138,9 @@ struct MatchArgs {
 // The seeding kernel comes in CTAs of up to kSeedThreads[i] threads, those of
 // 256 with fewer registers per thread or (wide) more; its instantiations are
 // spread over translation units that compile in parallel.
-constexpr int kSeedShapes = 4;
-constexpr int kSeedThreads[kSeedShapes] = {256, 256, 384, 512};
-constexpr bool kSeedWide[kSeedShapes] = {false, true, false, false};
+constexpr int kSeedShapes = 5;
+constexpr int kSeedThreads[kSeedShapes] = {256, 256, 384, 512, 1024};
+constexpr bool kSeedWide[kSeedShapes] = {false, true, false, false, false};
 typedef void (*SeedKernel)(const DevParams, const SeedArgs);
 // the instantiation for CTAs of `threads` threads, with the HLT2-style pass
 // loop (seq) or with the matching fused in
@@ -154,10 +159,12 @@ size_t match_smem_bytes(int velo_smem);
 // between them; k_gather always follows k_scan that way).  Their CTAs may
 // then wait on the SMs for that kernel, which only pays where no other
 // stream's kernels want those SMs.
-cudaError_t launch_build(const DevParams& P, const BuildArgs& a, int grid, int threads, cudaStream_t s,
-                         bool chained = true);
-cudaError_t launch_seed(const DevParams& P, const SeedArgs& a, int grid, int threads, bool wide, size_t smem, cudaStream_t s,
-                        bool chained = true);
+// started (may be null): recorded when all CTAs of the launch have begun.
+cudaError_t launch_build(const DevParams& P, const BuildArgs& a, int grid, int threads, cudaStream_t s);
+cudaError_t launch_build_large(const DevParams& P, const BuildArgs& a, int grid, cudaStream_t s, cudaEvent_t started);
+cudaError_t launch_order(const BuildArgs& a, cudaStream_t s, bool chained = true);
+cudaError_t launch_seed(const DevParams& P, const SeedArgs& a, int grid, int threads, bool wide, size_t smem,
+                        cudaStream_t s, bool chained = true, cudaEvent_t started = nullptr);
 cudaError_t launch_gather(const GatherArgs& a, cudaStream_t s, bool chained = true);
 cudaError_t launch_match(const DevParams& P, const MatchArgs& a, int grid, int threads, cudaStream_t s);
 

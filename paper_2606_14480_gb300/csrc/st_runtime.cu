@@ -386,18 +386,23 @@ bool derive_params(const st_config& c, DevParams& P, std::string& err) {
 
 namespace st {
 
+static SeedShape seed_shape(int threads, bool wide, int smem_hits, int velo_smem, bool bps) {
+    SeedShape s;
+    s.threads = threads;
+    s.wide = wide;
+    s.smem_hits = smem_hits;
+    s.tbl_smem = smem_hits / 2;
+    s.key_smem = std::max(64, smem_hits / 8);  // kept seeds whose UV keys and stereo x stay in shared memory
+    s.velo_smem = velo_smem;
+    s.smem = std::max(seed_smem_bytes(threads, smem_hits, s.tbl_smem, s.key_smem), match_smem_bytes(velo_smem));
+    s.bps = bps ? seed_blocks_per_sm(threads, wide, s.smem) : 0;
+    return s;
+}
+
 int seed_shapes(const st_config& c, SeedShape out[kSeedShapes], bool bps) {
     int n = 0;
     auto add = [&](int threads, bool wide, int smem_hits, int velo_smem) {
-        SeedShape& s = out[n++];
-        s.threads = threads;
-        s.wide = wide;
-        s.smem_hits = smem_hits;
-        s.tbl_smem = smem_hits / 2;
-        s.key_smem = std::max(64, smem_hits / 8);  // kept seeds whose UV keys and stereo x stay in shared memory
-        s.velo_smem = velo_smem;
-        s.smem = std::max(seed_smem_bytes(threads, smem_hits, s.tbl_smem, s.key_smem), match_smem_bytes(velo_smem));
-        s.bps = bps ? seed_blocks_per_sm(threads, wide, s.smem) : 0;
+        out[n++] = seed_shape(threads, wide, smem_hits, velo_smem, bps);
     };
     add(c.threads_seed, false, c.smem_hits, 512);
     if (c.threads_seed <= 256) add(256, true, std::max(c.smem_hits, 1536), 512);
@@ -445,7 +450,7 @@ struct Workspace {
     int build_ctas = 0, seed_ctas = 0;  // CTAs the per-CTA scratch is sized for
     // carved pointers
     // [0] build, [1] seed, [2] match queues; fused matching: [3] announced, [4] fault,
-    // [5] claimed, [6] done; [16, 144) item classes, [144, 272) their fill; then ev_done
+    // [5] claimed, [6] done; [7] costly items, [10] their queue; [16, 144) item classes, [144, 272) their fill; then ev_done
     int32_t* queues = nullptr;
     unsigned long long* pool_ctr = nullptr;
     float* cx = nullptr;
@@ -485,6 +490,9 @@ struct st_ctx {
     size_t match_smem = 0, build_smem_max = 0;
     SeedShape shape[kSeedShapes];  // [0] as configured, then the larger CTAs for batches that leave SMs idle
     int n_shapes = 0;
+    SeedShape big;                 // for the costliest items of a batch that may hold large events
+    cudaStream_t side = nullptr;   // their launches run beside the others'
+    cudaEvent_t ev_fork = nullptr, ev_started = nullptr, ev_join = nullptr;
     int match_bps = 0;
     Pipeline* pipe = nullptr;
     std::mutex pipe_mu;
@@ -493,6 +501,16 @@ struct st_ctx {
     int64_t wait_ns = kDefaultWaitNs;  // fused seeding kernel: longest wait for an announced event
     cudaEvent_t tev[4][2] = {};
     bool tused[4] = {};
+
+    // the side stream takes up after what s holds now; s goes on after both
+    cudaError_t fork(cudaStream_t s) {
+        const cudaError_t e = cudaEventRecord(ev_fork, s);
+        return e != cudaSuccess ? e : cudaStreamWaitEvent(side, ev_fork, 0);
+    }
+    cudaError_t join(cudaStream_t s) {
+        const cudaError_t e = cudaEventRecord(ev_join, side);
+        return e != cudaSuccess ? e : cudaStreamWaitEvent(s, ev_join, 0);
+    }
 };
 
 struct st_graph {
@@ -536,6 +554,9 @@ static void tmark(st_ctx* ctx, const Workspace& w, int k, int end, cudaStream_t 
 constexpr size_t kQueueBytes = 64 + 2 * 128 * sizeof(int32_t);
 constexpr int kBuildSmemHits = 6144;  // larger events keep their per-hit arrays in scratch
 constexpr int kBuildCtasPerSm = 8;
+constexpr int kBuildSplitHits = 4096;   // split batches: hits of an event built in the smaller CTAs
+constexpr int kBuildLargeHits = 16384;  // and hits and buckets that the larger ones keep in shared memory
+constexpr int kBuildLargeBins = 256;
 
 // buckets per container slot for a batch: about four hits per bucket (the
 // rank sort inside a bucket is quadratic but tiny; fewer buckets mean less
@@ -637,6 +658,12 @@ static int ensure(st_ctx* ctx, Workspace& w, int64_t ne, int64_t nh, int32_t mh,
 // context
 // ---------------------------------------------------------------------------
 
+static void destroy_side(st_ctx* ctx) {
+    for (cudaEvent_t ev : {ctx->ev_fork, ctx->ev_started, ctx->ev_join})
+        if (ev) cudaEventDestroy(ev);
+    if (ctx->side) cudaStreamDestroy(ctx->side);
+}
+
 extern "C" int st_create(const st_config* cfg, int device, st_ctx** out) {
     if (!cfg || !out) return ST_EINVAL;
     *out = nullptr;
@@ -676,12 +703,20 @@ extern "C" int st_create(const st_config* cfg, int device, st_ctx** out) {
     e = set_smem_limits(ctx->smem_optin);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->counters, sizeof(unsigned long long) * C_N);
     if (e == cudaSuccess) e = cudaMemset(ctx->counters, 0, sizeof(unsigned long long) * C_N);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking);
+    for (cudaEvent_t* ev : {&ctx->ev_fork, &ctx->ev_started, &ctx->ev_join})
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         if (ctx->counters) cudaFree(ctx->counters);
+        destroy_side(ctx);
         delete ctx;
         return ST_ECUDA;
     }
     ctx->n_shapes = seed_shapes(c, ctx->shape, true);
+    // 48 registers a thread: a smaller CTA still fits beside it (with 64, alone
+    // on its SM, the split batches above take 746 and 896 us; 768 threads 758
+    // and 893, 512 threads 814 and 946)
+    if (c.threads_seed <= 256) ctx->big = seed_shape(1024, false, 8192, 1024, true);
     ctx->match_bps = match_blocks_per_sm(c.threads_match, ctx->match_smem, c.final_sel != 0);
     *out = ctx;
     return ST_OK;
@@ -696,6 +731,7 @@ extern "C" void st_destroy(st_ctx* ctx) {
     cudaDeviceSynchronize();
     if (ctx->ws.base) cudaFree(ctx->ws.base);
     if (ctx->counters) cudaFree(ctx->counters);
+    destroy_side(ctx);
     for (int k = 0; k < 4; ++k)
         for (int j = 0; j < 2; ++j)
             if (ctx->tev[k][j]) cudaEventDestroy(ctx->tev[k][j]);
@@ -726,25 +762,38 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
     int rc = ensure(ctx, w, H.n_events, n_hits_total, H.max_hits_per_event, S.cap, may_alloc);
     if (rc != ST_OK) return rc;
     const st_config& c = ctx->cfg;
-    const int bins = bins_for(H.n_events, n_hits_total);
-    const int build_cap = std::min<int>(H.max_hits_per_event, kBuildSmemHits);
+    const SeedShape& sh = pick_seed_shape(ctx->shape, ctx->n_shapes, c, 2 * H.n_events, ctx->n_sms, w.seed_ctas);
+    const int sbps = c.ctas_per_sm > 0 ? std::min(std::max(1, sh.bps), c.ctas_per_sm) : std::max(1, sh.bps);
+    int g_seed = static_cast<int>(std::max<int64_t>(
+        1, std::min<int64_t>({2 * H.n_events, int64_t(ctx->n_sms) * sbps, int64_t(w.seed_ctas)})));
+    // every item has a CTA of its own from the start: no queue, no order
+    // A batch that may hold events many times the ordinary size waits for its
+    // largest items: one of 800 tracks took 1.1 ms in a CTA of 256 threads,
+    // 630 us in one of 512, and its container 82 us in scratch memory.  Such
+    // batches are split: their large events and costliest items go to larger
+    // CTAs (1024 threads, one per SM) in launches of their own on a side stream,
+    // and the others follow once those CTAs have begun, so that every SM takes
+    // one of each.  2000 events of 120 tracks on average, up to 800: 1286 us in
+    // one launch, 679 us split; 400 events of 500 tracks 938 and 820 us.  The
+    // line is the size from which containers leave the smaller CTAs' shared
+    // memory.  Not on the serving pipeline's slots, whose streams run beside
+    // each other already, and not below one item per SM, where 512 threads serve
+    // every item.
+    const bool split = &w == &ctx->ws && 2 * H.n_events > ctx->n_sms && c.ctas_per_sm == 0 && ctx->big.bps > 0 &&
+                       H.max_hits_per_event > kBuildSmemHits && w.seed_ctas >= 3 * ctx->n_sms;
+    const bool one_round = 2 * H.n_events <= g_seed && !split;
+    const int build_cap = std::min<int>(H.max_hits_per_event, split ? kBuildSplitHits : kBuildSmemHits);
+    const int bins = split ? bins_for(1, build_cap) : bins_for(H.n_events, n_hits_total);
     int bbps = std::max(1, build_blocks_per_sm(c.threads_build, build_smem_bytes(bins, build_cap)));
     if (c.ctas_per_sm > 0) bbps = std::min(bbps, c.ctas_per_sm);
     const int g_build = static_cast<int>(std::max<int64_t>(
         1, std::min<int64_t>({H.n_events, int64_t(ctx->n_sms) * bbps, int64_t(w.build_ctas)})));
-    const SeedShape& sh = pick_seed_shape(ctx->shape, ctx->n_shapes, c, 2 * H.n_events, ctx->n_sms, w.seed_ctas);
-    int sbps = std::max(1, sh.bps);
-    if (c.ctas_per_sm > 0) sbps = std::min(sbps, c.ctas_per_sm);
-    const int g_seed = static_cast<int>(std::max<int64_t>(
-        1, std::min<int64_t>({2 * H.n_events, int64_t(ctx->n_sms) * sbps, int64_t(w.seed_ctas)})));
     const bool fused = V && L;
     ST_CUDA(ctx, cudaMemsetAsync(w.queues, 0, kQueueBytes + (fused ? 2 * sizeof(int32_t) * size_t(H.n_events) : 0), s));
     if (H.n_events == 0) {
         ST_CUDA(ctx, cudaMemsetAsync(S.ev_off, 0, sizeof(int32_t), s));
         return ST_OK;
     }
-    // every item has a CTA of its own from the start: no queue, no order
-    const bool one_round = 2 * H.n_events <= g_seed;
     BuildArgs b;
     b.n_events = H.n_events;
     b.ev_off = H.ev_off;
@@ -777,7 +826,20 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
     const bool marks = ctx->timing && &w == &ctx->ws;
     const bool chain = &w == &ctx->ws;
     tmark(ctx, w, 0, 0, s);
-    ST_CUDA(ctx, launch_build(ctx->P, b, g_build, c.threads_build, s, chain));
+    if (split) {
+        b.split_hits = kBuildSplitHits;
+        b.n_big = w.queues + 7;
+        BuildArgs l = b;
+        l.smem_hits = std::min<int>(H.max_hits_per_event, kBuildLargeHits);
+        l.bins = std::min(bins_for(1, H.max_hits_per_event), kBuildLargeBins);
+        ST_CUDA(ctx, ctx->fork(s));
+        ST_CUDA(ctx, launch_build_large(ctx->P, l, static_cast<int>(std::min<int64_t>(H.n_events, ctx->n_sms)),
+                                        ctx->side, ctx->ev_started));
+        ST_CUDA(ctx, cudaStreamWaitEvent(s, ctx->ev_started, 0));
+    }
+    ST_CUDA(ctx, launch_build(ctx->P, b, g_build, c.threads_build, s));
+    if (split) ST_CUDA(ctx, ctx->join(s));
+    ST_CUDA(ctx, launch_order(b, s, chain && !split));
     tmark(ctx, w, 0, 1, s);
 
     SeedArgs a;
@@ -816,7 +878,7 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
         // finishing times; with one item each there is nothing to even out, and
         // the waiting CTAs slow the others down (250 Run-3-like events: 117 us
         // with it, 107 without).  A wait limit of 0 asks for the waits' timeout.
-        a.defer_match = defer && (!one_round || ctx->wait_ns == 0) ? 1 : 0;
+        a.defer_match = defer && !split && (!one_round || ctx->wait_ns == 0) ? 1 : 0;
         a.ev_done = w.ev_done;
         a.ready = w.ev_done + H.n_events;
         a.ready_ctr = w.queues + 3;
@@ -829,7 +891,27 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
         if (ctx->timing && &w == &ctx->ws) ctx->tused[3] = false;  // matching runs inside k_seed
     }
     tmark(ctx, w, 1, 0, s);
-    ST_CUDA(ctx, launch_seed(ctx->P, a, g_seed, sh.threads, sh.wide, sh.smem, s, chain && !marks));
+    if (split) {
+        const SeedShape& big = ctx->big;
+        const int g_big = static_cast<int>(std::min<int64_t>(2 * H.n_events, ctx->n_sms));
+        SeedArgs l = a;
+        l.smem_hits = big.smem_hits;
+        l.tbl_smem = big.tbl_smem;
+        l.key_smem = big.key_smem;
+        l.velo_smem = fused ? big.velo_smem : 0;
+        l.part = 1;
+        l.n_big = b.n_big;
+        l.queue = w.queues + 10;
+        ST_CUDA(ctx, ctx->fork(s));
+        ST_CUDA(ctx, launch_seed(ctx->P, l, g_big, big.threads, big.wide, big.smem, ctx->side, false, ctx->ev_started));
+        ST_CUDA(ctx, cudaStreamWaitEvent(s, ctx->ev_started, 0));
+        a.part = 2;
+        a.n_big = b.n_big;
+        a.slot += g_big * w.slot_stride;
+        g_seed = std::min(g_seed, w.seed_ctas - g_big);
+    }
+    ST_CUDA(ctx, launch_seed(ctx->P, a, g_seed, sh.threads, sh.wide, sh.smem, s, chain && !marks && !split));
+    if (split) ST_CUDA(ctx, ctx->join(s));
     tmark(ctx, w, 1, 1, s);
 
     GatherArgs g;
@@ -855,7 +937,7 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
         g.chi2 = L->chi2;
     }
     tmark(ctx, w, 2, 0, s);
-    ST_CUDA(ctx, launch_gather(g, s, chain && !marks));
+    ST_CUDA(ctx, launch_gather(g, s, chain && !marks && !split));
     tmark(ctx, w, 2, 1, s);
     return ST_OK;
 }

@@ -28,7 +28,7 @@ size_t seed_slot_limit_bytes(int cand_cap, int max_xhits) {
 SeedKernel seed_kernel(int threads, bool wide, bool seq, bool fused) {
     return threads <= 256 ? (wide ? seed_kernel_256w(seq, fused) : seed_kernel_256(seq, fused))
            : threads <= 384 ? seed_kernel_384(seq, fused)
-                            : seed_kernel_512(seq, fused);
+           : threads <= 512 ? seed_kernel_512(seq, fused) : seed_kernel_1024(seq, fused);
 }
 
 }  // namespace st

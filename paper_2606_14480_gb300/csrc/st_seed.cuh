@@ -32,10 +32,12 @@ constexpr int kSeedRegs256 = 48;
 constexpr int kSeedRegs256w = 64;
 constexpr int kSeedRegs384 = 56;
 constexpr int kSeedRegs512 = 64;
+constexpr int kSeedRegs1024 = 48;  // leaves room for a smaller CTA beside it
 SeedKernel seed_kernel_256(bool seq, bool fused);
 SeedKernel seed_kernel_256w(bool seq, bool fused);
 SeedKernel seed_kernel_384(bool seq, bool fused);
 SeedKernel seed_kernel_512(bool seq, bool fused);
+SeedKernel seed_kernel_1024(bool seq, bool fused);
 
 // ---------------------------------------------------------------------------
 // per-zone hit maps: one bit per 2 mm bin that holds a hit, and per word of 32
@@ -1141,7 +1143,7 @@ k_seed(const __grid_constant__ DevParams P, const __grid_constant__ SeedArgs A) 
         __syncthreads();
         if (tid == 0) {
             V.match = -1;
-            const int n2 = A.n_list ? *A.n_list : static_cast<int>(2 * A.n_events);
+            const int n2 = A.part == 1 ? *A.n_big : A.n_list ? *A.n_list : static_cast<int>(2 * A.n_events);
             if (kFuse && fin >= 0 && atomicAdd(A.ev_done + fin, 1) == 1) {
                 // this CTA finished the event's second half (the other half's
                 // records were released before its count; the fence orders
@@ -1158,7 +1160,7 @@ k_seed(const __grid_constant__ DevParams P, const __grid_constant__ SeedArgs A) 
                 atomicAdd(A.done_ctr, 1);
             }
             if (V.match < 0) {
-                const int q = A.order ? atomicAdd(A.queue, 1) : first ? static_cast<int>(blockIdx.x) : n2;
+                const int q = A.order ? (A.part == 2 ? *A.n_big : 0) + atomicAdd(A.queue, 1) : first ? static_cast<int>(blockIdx.x) : n2;
                 first = false;
                 if (q < n2) {
                     V.item = A.order ? A.order[q] : q;

@@ -226,6 +226,7 @@ extern "C" int seeding_run_static(const st_config* cfg, const st_hits* H, st_see
     ba.queue = queues + 0;
     ba.counters = counters;
     e = launch_build(P, ba, g_build, cfg->threads_build, s);
+    if (e == cudaSuccess) e = launch_order(ba, s);
     if (e != cudaSuccess) return fail(err, err_len, ST_ECUDA, "k_build: %s", cudaGetErrorString(e));
 
     SeedArgs sa;

@@ -75,6 +75,67 @@ def test_larger_ctas_give_the_same(mode, items, zmx):
     assert n > 0
 
 
+def _concat(parts):
+    """One batch of (events, hits kept of each or None) pairs."""
+    x, zone, velo, eo, vo = [], [], [], [0], [0]
+    for b, keep in parts:
+        for e in range(b.n_events):
+            h0, h1 = int(b.ev_off[e]), int(b.ev_off[e + 1])
+            h1 = h1 if keep is None else h0 + keep
+            assert h1 <= b.ev_off[e + 1]
+            x.append(b.x[h0:h1])
+            zone.append(b.zone[h0:h1])
+            velo.append(b.velo[b.velo_off[e]:b.velo_off[e + 1]])
+            eo.append(eo[-1] + h1 - h0)
+            vo.append(vo[-1] + len(velo[-1]))
+    return np.array(eo), np.concatenate(x), np.concatenate(zone), np.array(vo), np.concatenate(velo)
+
+
+@pytest.mark.parametrize("mode", [{}, dict(uv_mode=1), dict(iter_mode=1)], ids=["hlt1", "hough", "seq"])
+def test_large_events_beside_ordinary(mode, zmx):
+    """Batches that may hold large events: those events' containers and items
+    run in larger CTAs beside the others.  Around the sizes that divide them,
+    with a faulty large event and one above the bound, the results are those of
+    the launches without the division (a set ctas_per_sm)."""
+    d = make_events(2, seed=4021, tracks=("fixed", 500))
+    g = make_events(1, seed=4022, tracks=("fixed", 1300))
+    assert np.diff(d.ev_off).min() > 6144 and np.diff(g.ev_off).min() > 16385
+    s = make_events(130, seed=4023, tracks=("fixed", 25))
+    eo, x, zone, vo, velo = _concat([(s, None), (d, 4096), (s.subset(range(9)), 0), (d, 4097), (d, None), (g, 16384),
+                                     (d, 6144), (g, 16385), (d, None), (s, None)])
+    last = 130 + 2 + 9 + 2 + 2 + 1 + 2 + 1  # the first of the two large events after the 16385-hit one
+    zone = zone.copy()
+    zone[eo[last] + 5000] = 24
+    cap = 80 * (len(eo) - 1)
+    for mh in (16385, 16384):
+        res = []
+        for shape in (dict(ctas_per_sm=8), {}):
+            _, gcfg = parity.config_pair(zmx, cand_cap=16384, **mode, **shape)
+            db = st.DeviceBatch(eo, x, zone, vo, velo, max_hits=mh)
+            ctx = st.Context(gcfg)
+            res.append(st.run_batch(ctx, db, cap=cap).to_numpy())
+            if not mode and not shape:
+                out = st.DeviceOutputs(len(eo) - 1, cap)
+                gr = ctx.st_graph_create(db.hits, db.velo_s, out.seeds, out.long)
+                gr.st_graph_launch()
+                gr.st_graph_launch()
+                torch.cuda.synchronize()
+                res.append(out.to_numpy())
+                gr.close()
+            ctx.close()
+        want = np.zeros(len(eo) - 1, np.int32)
+        want[last] = st.ST_EINVAL
+        want[np.diff(eo) > mh] = st.ST_OVERFLOW
+        for r in res:
+            # (the HLT2-style mode stores all UV combinations of an item and
+            # refuses those whose store runs over)
+            full = (r["status"] == st.ST_OVERFLOW) & (np.diff(eo) > 6144) if mode.get("iter_mode") else False
+            assert np.array_equal(r["status"], np.where(full, st.ST_OVERFLOW, want))
+            assert r["ev_off"][-1] > 1000
+            for k in KEYS:
+                assert np.array_equal(r[k], res[0][k]), (mh, k)
+
+
 @pytest.mark.parametrize("n,tracks,over", [
     (60, 150, {}),                                       # one CTA per item
     (20, 260, {}),                                       # halves with more hits than shared memory holds
