@@ -560,6 +560,7 @@ k_match(const __grid_constant__ DevParams P, const __grid_constant__ MatchArgs A
         e = s_item;
         __syncthreads();
     }
+    pdl_signal();
     flush_counters(A.counters + C_MATCH_PAIRS, ctr, 3);
     flush_counters(A.counters + C_MATCH_EVAL, ctr + 3, 1);
 }
@@ -620,31 +621,6 @@ int match_blocks_per_sm(int threads, size_t smem, bool final_sel) {
     else
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_match<false>, threads, smem);
     return n;
-}
-
-// A launch as a programmatic dependent of the stream's previous kernel
-// (chained), or a plain one; `started` (if given) is recorded when all its
-// CTAs have begun.
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_k(void (*k)(KArgs...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s,
-                            bool chained, cudaEvent_t started, Args&&... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[2];
-    cfg.attrs = at;
-    if (chained) {
-        at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
-    }
-    if (started) {
-        at[cfg.numAttrs].id = cudaLaunchAttributeLaunchCompletionEvent;
-        at[cfg.numAttrs].val.launchCompletionEvent.event = started;
-        at[cfg.numAttrs++].val.launchCompletionEvent.flags = 0;
-    }
-    return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
 }
 
 cudaError_t launch_build(const DevParams& P, const BuildArgs& a, int grid, int threads, cudaStream_t s) {

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cstdint>
+#include <utility>
 #include <cuda_runtime.h>
 
 #include "st_device.cuh"
@@ -167,6 +168,31 @@ cudaError_t launch_seed(const DevParams& P, const SeedArgs& a, int grid, int thr
                         cudaStream_t s, bool chained = true, cudaEvent_t started = nullptr);
 cudaError_t launch_gather(const GatherArgs& a, cudaStream_t s, bool chained = true);
 cudaError_t launch_match(const DevParams& P, const MatchArgs& a, int grid, int threads, cudaStream_t s);
+
+// A launch as a programmatic dependent of the stream's previous kernel
+// (chained), or a plain one; `started` (if given) is recorded when all its
+// CTAs have begun.
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_k(void (*k)(KArgs...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s,
+                            bool chained, cudaEvent_t started, Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    cfg.attrs = at;
+    if (chained) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (started) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeLaunchCompletionEvent;
+        at[cfg.numAttrs].val.launchCompletionEvent.event = started;
+        at[cfg.numAttrs++].val.launchCompletionEvent.flags = 0;
+    }
+    return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
+}
 
 // occupancy helpers
 int build_blocks_per_sm(int threads, size_t smem);

@@ -1080,8 +1080,12 @@ extern "C" int ut_run(st_ctx* ctx, const st_velo* velo, const st_seeds* seeds, c
     a.ut_hits = uo->hits;
     a.ut_n = uo->n_hits;
     a.gamma = uo->gamma;
-    const int grid = static_cast<int>(std::min<int64_t>(ut->n_events, int64_t(ctx->n_sms) * 6));
-    ST_CUDA(ctx, launch_ut(U, a, grid, static_cast<cudaStream_t>(stream)));
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    ST_CUDA(ctx, cudaStreamIsCapturing(s, &cs));
+    // a programmatic dependent of what the stream holds (1.5 us less after
+    // k_match); not in a capture, where that may be more than a kernel
+    ST_CUDA(ctx, launch_ut(U, a, ctx->n_sms, s, cs == cudaStreamCaptureStatusNone));
     return ST_OK;
 }
 

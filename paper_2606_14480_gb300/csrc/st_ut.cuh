@@ -37,6 +37,7 @@ struct UtArgs {
     float* gamma;            // [seeds]
 };
 
-cudaError_t launch_ut(const UtParams& U, const UtArgs& a, int grid, cudaStream_t s);
+// chained: as a programmatic dependent of the stream's previous kernel
+cudaError_t launch_ut(const UtParams& U, const UtArgs& a, int n_sms, cudaStream_t s, bool chained);
 
 }  // namespace st

@@ -1,0 +1,81 @@
+"""The UT search at the edges of its layout: hits around what shared memory
+holds and batches of several rounds."""
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import oracle  # noqa: E402
+import parity  # noqa: E402
+from conftest import workload  # noqa: E402
+from paper_2606_14480_gb300 import st  # noqa: E402
+from synth import calibrate_zmatch  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def zmx():
+    return calibrate_zmatch(7826.0)
+
+
+@pytest.mark.parametrize("nu", [0, 1, 767, 768, 769, 4096, 4097])
+def test_ut_sizes(nu, zmx):
+    """UT hits of an event around the threads' shares and shared memory."""
+    b = workload("run3", n_events=6)
+    ocfg, gcfg = parity.config_pair(zmx)
+    rng = np.random.default_rng(4103)
+    ux, ul = [], []
+    for e in range(b.n_events):
+        x, l = b.ut_of(e)
+        more = max(nu - len(x), 0)
+        ux.append(np.concatenate([x, rng.uniform(-1500, 1500, more).astype(np.float32)])[:nu])
+        ul.append(np.concatenate([l, rng.integers(0, 4, more).astype(np.int32)])[:nu])
+    db = st.DeviceBatch(b.ev_off, b.x, b.zone, b.velo_off, b.velo)
+    db.add_ut(np.arange(b.n_events + 1) * nu, np.concatenate(ux), np.concatenate(ul))
+    ctx = st.Context(gcfg)
+    out = st.run_batch(ctx, db)
+    pre = out.velo_idx.cpu().numpy().copy()
+    ctx.ut_run(db.velo_s, out.seeds, db.ut, out.long, out.ut_out)
+    r = out.to_numpy()
+    ctx.close()
+    for e in range(b.n_events):
+        s0, s1 = int(r["ev_off"][e]), int(r["ev_off"][e + 1])
+        w = oracle.ut_search(ocfg, b.velo_of(e), r["state"][s0:s1], pre[s0:s1], ux[e], ul[e], ledger_tau=1e-4)
+        led = w["ledger"]
+        near = {int(h[0]) for h in led[led["margin"] <= parity.TAU]["hits"]} if len(led) else set()
+        for k in range(s1 - s0):
+            if pre[s0 + k] >= 0 and k not in near:
+                assert np.array_equal(r["ut_hits"][s0 + k], w["ut_hits"][k]), (e, k)
+                assert r["velo_idx"][s0 + k] == w["velo_idx"][k]
+
+
+def test_ut_rounds(zmx):
+    """More events than CTAs at once: each event's hits are those it gets in a
+    small batch."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    one = workload("run3", n_events=40)
+    reps = (8 * sms + 3) // 40 + 2
+    _, gcfg = parity.config_pair(zmx)
+    res = []
+    for n in (1, reps):
+        db = st.DeviceBatch(*[np.concatenate([[0]] + [o[1:] + k * o[-1] for k in range(n)]) if i in (0, 3) else
+                              np.concatenate([o] * n) for i, o in
+                              enumerate((one.ev_off, one.x, one.zone, one.velo_off, one.velo))])
+        db.add_ut(np.concatenate([[0]] + [one.ut_off[1:] + k * one.ut_off[-1] for k in range(n)]),
+                  np.concatenate([one.ut_x] * n), np.concatenate([one.ut_layer] * n))
+        ctx = st.Context(gcfg)
+        out = st.run_batch(ctx, db)
+        ctx.ut_run(db.velo_s, out.seeds, db.ut, out.long, out.ut_out)
+        res.append(out.to_numpy())
+        ctx.close()
+    a, b = res
+    n = int(a["ev_off"][-1])
+    assert n > 0 and int(b["ev_off"][-1]) == n * reps
+    for k in ("ut_hits", "ut_n", "ut_gamma", "velo_idx", "chi2"):
+        for q in range(reps):
+            assert np.array_equal(b[k][q * n:(q + 1) * n], a[k][:n]), (k, q)
+    assert np.array_equal(b["n_long"], np.tile(a["n_long"], reps))
