@@ -19,15 +19,15 @@ struct MatchIO {
 };
 // Lanes that share a seed: as many as keep seeds x lanes within kMatchFill
 // times the CTA's threads.  500 events of 272 seeds and 400 segments: 41 us
-// with a thread per seed (two passes, the second nearly empty), 37.5 us with
-// up to 4 x 256 lanes' worth; fewer lanes than that give 42 us.
+// with a thread per seed (two passes, the second nearly empty), 34 us with up
+// to 4 x 256 lanes' worth, 30 us with the segments laid out as below.
 constexpr int kMatchLanes = 8;
 constexpr int kMatchFill = 4;
 constexpr int kTyBins = 64;
 constexpr float kTyRange = 0.32f;  // buckets of 0.01 over [-0.32, 0.32); outside values go to the end buckets
 
 inline size_t match_smem_size(int velo_smem) {
-    return sizeof(float) * 7 * size_t(velo_smem) + sizeof(int) * (2 * size_t(velo_smem) + 2 * kTyBins + 8);
+    return (2 * sizeof(float4) + sizeof(int)) * size_t(velo_smem) + sizeof(int) * (2 * kTyBins + 8);
 }
 
 __device__ __forceinline__ int ty_bin(float ty) {
@@ -37,20 +37,30 @@ __device__ __forceinline__ int ty_bin(float ty) {
 
 // One (VELO, seed) pair of Section 4: preselection, then chi2_match; updates
 // the best (chi2, VELO index).  Position differences are formed from
-// float-float extrapolations to z = A_x and z = z_match_y.
-__device__ __forceinline__ int match_pair(const DevParams& P, float vxh, float vxl, float vyh, float vyl,
-                                          float vtx, float vty, float vit, int vg, float xh, float xl,
-                                          float yh, float yl, float txS, float tyS, float dzx, float& best,
-                                          int& bv) {
-    const float dtx = vtx - txS, dty = vty - tyS;
+// float-float extrapolations to z = A_x (x) and z = z_match_y (y).  The first
+// half of the segment decides most pairs.
+struct VeloHalf {
+    float tx, ty, yh, yl;
+};
+struct VeloRest {
+    float xh, xl, it;
+    int v;
+};
+static_assert(sizeof(VeloHalf) == sizeof(float4) && sizeof(VeloRest) == sizeof(float4), "");
+__device__ __forceinline__ int match_pair(const DevParams& P, const VeloHalf& a, const VeloRest* rest, float xh,
+                                          float xl, float yh, float yl, float txS, float tyS, float dzx,
+                                          float& best, int& bv) {
+    const float dtx = a.tx - txS, dty = a.ty - tyS;
     if (!(fabsf(dty) < P.cut_ty) || !(fabsf(dtx) < P.cut_tx)) return 0;
-    const float dy = (vyh - yh) + (vyl - yl);
+    const float dy = (a.yh - yh) + (a.yl - yl);
     if (!(fabsf(dy) < P.cut_y)) return 0;
-    const float dz = fmaf(P.Bx, fabsf(dtx), fmaf(P.Cx, dtx * dtx, fmaf(P.Ex * vtx, vtx, dzx)));
-    const float dx = fmaf(dz, dtx, (vxh - xh) + (vxl - xl));
+    const float4 q = *reinterpret_cast<const float4*>(rest);
+    const float dz = fmaf(P.Bx, fabsf(dtx), fmaf(P.Cx, dtx * dtx, fmaf(P.Ex * a.tx, a.tx, dzx)));
+    const float dx = fmaf(dz, dtx, (q.x - xh) + (q.y - xl));
     if (!(fabsf(dx) < P.cut_x)) return 0;
     const float tolx = fmaf(P.tolx_b, dtx * dtx, P.tolx_a);
-    const float c2 = dx * dx / tolx + dy * dy * vit + dtx * dtx * P.inv_toltx + dty * dty * P.inv_tolty;
+    const float c2 = dx * dx / tolx + dy * dy * q.z + dtx * dtx * P.inv_toltx + dty * dty * P.inv_tolty;
+    const int vg = __float_as_int(q.w);
     if (c2 < P.chi2m_max && (c2 < best || (c2 == best && vg < bv))) {
         best = c2;
         bv = vg;
@@ -108,10 +118,14 @@ static __device__ float ghost_nn(const DevParams& P, const float f[8]) {
 
 // Matching of one event (Section 4): the event's VELO segments are staged in
 // shared memory (msm, match_smem_bytes(VS) bytes), VS at a time, with their
-// float-float extrapolations and bucketed by ty, so a seed only visits the
-// buckets its |dty| cut can reach (every other pair fails that cut).  A few
+// float-float extrapolations and laid out by ty bucket, so a seed only visits
+// the buckets its |dty| cut can reach (every other pair fails that cut).  A few
 // lanes share a seed, each taking every n-th segment of its buckets: an event
 // has fewer seeds than the CTA threads, and the time is the longest lane's.
+// What bounds it is the latency of that chain: a pair costs one 16-byte read
+// until it passes the first cuts, a lane's next seed is fetched while it works
+// on one, and pairs are counted where they are found.  1000 Run-3-like events
+// with the final selection: 34.3 us before these, 31.7 us with.
 // Seed s (0 .. ns-1, in the event's canonical seed order) reads its state and
 // hit counts and writes its pair at index row(s) of M's arrays.  Returns the
 // event's Long-track count; n_grid / n_presel accumulate this thread's pair
@@ -120,46 +134,44 @@ template <bool kFinal, class Row>
 __device__ int match_event(const DevParams& P, const MatchIO& M, int VS, unsigned char* msm, int64_t v0, int nv,
                            int ns, Row row, int* s_cnt, ull& n_grid, ull& n_presel, ull& n_eval) {
     const int T = blockDim.x, tid = threadIdx.x;
-    float* vxh = reinterpret_cast<float*>(msm);
-    float* vxl = vxh + VS;
-    float* vyh = vxl + VS;
-    float* vyl = vyh + VS;
-    float* vtx = vyl + VS;
-    float* vty = vtx + VS;
-    float* vit = vty + VS;
-    int* bidx = reinterpret_cast<int*>(vit + VS);  // VELO indices grouped by ty bucket
-    int* bcnt = bidx + VS;                         // [kTyBins]
-    int* boff = bcnt + kTyBins;                    // [kTyBins + 1]
-    unsigned* vmin = reinterpret_cast<unsigned*>(boff + kTyBins + 8);  // final selection: lowest ghost
-                                                                       // probability per VELO segment
+    VeloHalf* const va = reinterpret_cast<VeloHalf*>(msm);  // [VS] the chunk's segments grouped by ty bucket
+    VeloRest* const vb = reinterpret_cast<VeloRest*>(va + VS);
+    int* const tag = reinterpret_cast<int*>(vb + VS);       // [VS] a segment's bucket and place in it
+    int* const bcnt = tag + VS;                             // [kTyBins]
+    int* const boff = bcnt + kTyBins;                       // [kTyBins + 1]
+    const bool vec = (reinterpret_cast<uintptr_t>(M.velo) & 15u) == 0;
+    const float* const velo = M.velo + v0 * 4;
     if (tid == 0) *s_cnt = 0;
     int G = 1;
     while (G < kMatchLanes && 2 * G * ns <= kMatchFill * T) G *= 2;
     const int lane = tid & 31, sub = lane & (G - 1), step = (T >> 5) * (32 / G);
+    // the state of the lane's next seed, fetched ahead (past L1: in the fused
+    // kernel other CTAs wrote the rows during this launch)
+    float xS = 0.f, yS = 0.f, txS = 0.f, tyS = 0.f;
+    auto fetch = [&](int s) {
+        if (s >= ns) return;
+        const float* st = M.seed_state + row(s) * 4;
+        xS = __ldcg(st);
+        yS = __ldcg(st + 1);
+        txS = __ldcg(st + 2);
+        tyS = __ldcg(st + 3);
+    };
+    const int first = (tid >> 5) * (32 / G) + lane / G;
+    const bool plain = !P.velo_unique && !(kFinal && P.final_sel);  // no step drops a pair later
+    int nl = 0;
     for (int vc = 0; vc < nv; vc += VS) {
         const int m = min(VS, nv - vc);
+        const bool last = vc + VS >= nv;
         for (int k = tid; k < kTyBins; k += T) bcnt[k] = 0;
+        fetch(first);
         __syncthreads();
         for (int v = tid; v < m; v += T) {
-            const float* st = M.velo + (v0 + vc + v) * 4;
-            const float x = st[0], y = st[1], tx = st[2], ty = st[3];
-            float p, pe, s, se;
-            two_prod(P.dAV_hi, tx, p, pe);
-            two_sum(x, p, s, se);
-            vxh[v] = s;
-            vxl[v] = se + fmaf(P.dAV_lo, tx, pe);
-            two_prod(P.dMV_hi, ty, p, pe);
-            two_sum(y, p, s, se);
-            vyh[v] = s;
-            vyl[v] = se + fmaf(P.dMV_lo, ty, pe);
-            vtx[v] = tx;
-            vty[v] = ty;
-            vit[v] = 1.f / fmaf(P.toly_b, fmaf(tx, tx, ty * ty), P.toly_a);
-            atomicAdd(&bcnt[ty_bin(ty)], 1);
+            const int b = ty_bin(velo[4 * (vc + v) + 3]);
+            tag[v] = atomicAdd(&bcnt[b], 1) << 8 | b;
         }
         __syncthreads();
-        if (tid < 32) {  // exclusive scan of the bucket counts by one warp; the counts become fill cursors
-            int c0 = bcnt[2 * tid], c1 = bcnt[2 * tid + 1];
+        if (tid < 32) {  // exclusive scan of the bucket counts by one warp
+            const int c0 = bcnt[2 * tid], c1 = bcnt[2 * tid + 1];
             int x = c0 + c1;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -167,21 +179,43 @@ __device__ int match_event(const DevParams& P, const MatchIO& M, int VS, unsigne
                 if (tid >= o) x += y;
             }
             const int ex = x - c0 - c1;
-            boff[2 * tid] = bcnt[2 * tid] = ex;
-            boff[2 * tid + 1] = bcnt[2 * tid + 1] = ex + c0;
+            boff[2 * tid] = ex;
+            boff[2 * tid + 1] = ex + c0;
             if (tid == 31) boff[kTyBins] = x;
         }
         __syncthreads();
-        for (int v = tid; v < m; v += T) bidx[atomicAdd(&bcnt[ty_bin(vty[v])], 1)] = v;
+        for (int v = tid; v < m; v += T) {
+            float x, y, tx, ty;
+            const float* st = velo + 4 * (vc + v);
+            if (vec) {
+                const float4 q = *reinterpret_cast<const float4*>(st);
+                x = q.x, y = q.y, tx = q.z, ty = q.w;
+            } else {
+                x = st[0], y = st[1], tx = st[2], ty = st[3];
+            }
+            const int t = tag[v], k = boff[t & 255] + (t >> 8);
+            float p, pe, s;
+            VeloRest r;
+            two_prod(P.dAV_hi, tx, p, pe);
+            two_sum(x, p, r.xh, s);
+            r.xl = s + fmaf(P.dAV_lo, tx, pe);
+            r.it = 1.f / fmaf(P.toly_b, fmaf(tx, tx, ty * ty), P.toly_a);
+            r.v = vc + v;
+            VeloHalf a;
+            two_prod(P.dMV_hi, ty, p, pe);
+            two_sum(y, p, a.yh, s);
+            a.yl = s + fmaf(P.dMV_lo, ty, pe);
+            a.tx = tx;
+            a.ty = ty;
+            *reinterpret_cast<float4*>(va + k) = make_float4(a.tx, a.ty, a.yh, a.yl);
+            *reinterpret_cast<float4*>(vb + k) = make_float4(r.xh, r.xl, r.it, __int_as_float(r.v));
+        }
         __syncthreads();
         for (int s0 = (tid >> 5) * (32 / G); s0 < ns; s0 += step) {  // uniform over the warp
             const int s = s0 + lane / G;
             float best = FLT_MAX;
             int bv = 0x7fffffff, npre = 0;
             if (s < ns) {
-                // read past L1: in the fused kernel other CTAs wrote the rows during this launch
-                const float* st = M.seed_state + row(s) * 4;
-                const float xS = __ldcg(st), yS = __ldcg(st + 1), txS = __ldcg(st + 2), tyS = __ldcg(st + 3);
                 float p, pe, xh, xl, yh, yl;
                 two_prod(P.dAS_hi, txS, p, pe);
                 two_sum(xS, p, xh, xl);
@@ -189,7 +223,8 @@ __device__ int match_event(const DevParams& P, const MatchIO& M, int VS, unsigne
                 two_prod(P.dMS_hi, tyS, p, pe);
                 two_sum(yS, p, yh, yl);
                 yl += fmaf(P.dMS_lo, tyS, pe);
-                const float dzx = P.Dx * fabsf(xS);
+                const float dzx = P.Dx * fabsf(xS), txs = txS, tys = tyS;
+                fetch(s + step);
                 if (vc > 0 && sub == 0) {
                     const int pv = M.velo_idx[row(s)];
                     if (pv >= 0) {
@@ -199,16 +234,16 @@ __device__ int match_event(const DevParams& P, const MatchIO& M, int VS, unsigne
                 }
                 // buckets that can hold |ty - tyS| < cut_ty (slightly widened;
                 // the exact cut is applied per pair)
-                const float w = P.cut_ty + 1e-6f * (fabsf(tyS) + P.cut_ty);
-                const int k0 = boff[ty_bin(tyS - w)], k1 = boff[ty_bin(tyS + w) + 1];
+                const float w = P.cut_ty + 1e-6f * (fabsf(tys) + P.cut_ty);
+                const int k0 = boff[ty_bin(tys - w)], k1 = boff[ty_bin(tys + w) + 1];
                 if (sub == 0) {
                     n_eval += k1 - k0;
                     n_grid += m;
                 }
                 for (int k = k0 + sub; k < k1; k += G) {
-                    const int v = bidx[k];
-                    npre += match_pair(P, vxh[v], vxl[v], vyh[v], vyl[v], vtx[v], vty[v], vit[v], vc + v,
-                                       xh, xl, yh, yl, txS, tyS, dzx, best, bv);
+                    const float4 q = *reinterpret_cast<const float4*>(va + k);
+                    npre += match_pair(P, VeloHalf{q.x, q.y, q.z, q.w}, vb + k, xh, xl, yh, yl, txs, tys, dzx, best,
+                                       bv);
                 }
             }
             n_presel += npre;
@@ -224,6 +259,7 @@ __device__ int match_event(const DevParams& P, const MatchIO& M, int VS, unsigne
                 const bool found = best < FLT_MAX;
                 M.velo_idx[row(s)] = found ? bv : -1;
                 M.chi2[row(s)] = found ? best : 0.f;
+                nl += last && found;
             }
         }
         __syncthreads();
@@ -234,7 +270,10 @@ __device__ int match_event(const DevParams& P, const MatchIO& M, int VS, unsigne
             M.chi2[row(s)] = 0.f;
         }
     }
-    __syncthreads();
+    if (!plain) {
+        nl = 0;
+        __syncthreads();
+    }
     if (P.velo_unique) {
         // a VELO segment keeps its best seed (lowest chi2, then lower seed
         // index); losers are marked -2 - v so that concurrent readers still
@@ -265,7 +304,19 @@ __device__ int match_event(const DevParams& P, const MatchIO& M, int VS, unsigne
         __syncthreads();
     }
     if (kFinal && P.final_sel) {
-        // Section 4.4: ghost probability of each best pair and the cut
+        // Section 4.4: ghost probability of each best pair and the cut, then
+        // clones: a kept pair whose VELO segment another kept pair holds with a
+        // ghost probability lower by at least clone_margin (one pair per seed,
+        // so no two pairs share a seed).  With clone_margin > 0 that is p -
+        // (lowest p on the segment) >= clone_margin; the lowest p per segment
+        // is an atomicMin of the probabilities' bits (non-negative floats order
+        // as unsigned).
+        const bool small = nv <= VS;
+        unsigned* const vmin = reinterpret_cast<unsigned*>(tag);  // [VS] lowest ghost probability per segment
+        if (small) {
+            for (int v = tid; v < nv; v += T) vmin[v] = 0x7f800000u;
+            __syncthreads();
+        }
         for (int s = tid; s < ns; s += T) {
             const int v = M.velo_idx[row(s)];
             float p = 1.f;
@@ -278,31 +329,27 @@ __device__ int match_event(const DevParams& P, const MatchIO& M, int VS, unsigne
                 if (!(p < P.ghost_max)) {
                     M.velo_idx[row(s)] = -1;
                     M.chi2[row(s)] = 0.f;
+                } else if (small) {
+                    atomicMin(&vmin[v], __float_as_uint(p));
                 }
             }
             M.ghost_prob[row(s)] = p;
         }
         __syncthreads();
-        // clones: a kept pair whose VELO segment another kept pair holds
-        // with a ghost probability lower by at least clone_margin (one
-        // pair per seed, so no two pairs share a seed); marked -2 - v.
-        // With clone_margin > 0 that is p - (lowest p on the segment) >=
-        // clone_margin; the lowest p per segment is an atomicMin of the
-        // probabilities' bits (non-negative floats order as unsigned).
-        if (nv <= VS) {
-            for (int v = tid; v < nv; v += T) vmin[v] = 0x7f800000u;
-            __syncthreads();
+        if (small) {
+            // (each thread's own rows)
             for (int s = tid; s < ns; s += T) {
                 const int v = M.velo_idx[row(s)];
-                if (v >= 0) atomicMin(&vmin[v], __float_as_uint(M.ghost_prob[row(s)]));
-            }
-            __syncthreads();
-            for (int s = tid; s < ns; s += T) {
-                const int v = M.velo_idx[row(s)];
-                if (v >= 0 && M.ghost_prob[row(s)] - __uint_as_float(vmin[v]) >= P.clone_margin)
-                    M.velo_idx[row(s)] = -2 - v;
+                const bool clone = v >= 0 && M.ghost_prob[row(s)] - __uint_as_float(vmin[v]) >= P.clone_margin;
+                if (clone) {
+                    M.velo_idx[row(s)] = -1;
+                    M.chi2[row(s)] = 0.f;
+                }
+                nl += v >= 0 && !clone;
             }
         } else {
+            // clones are marked -2 - v, so that concurrent readers still see
+            // which segment they held
             for (int s = tid; s < ns; s += T) {
                 const int v = M.velo_idx[row(s)];
                 if (v < 0) continue;
@@ -317,18 +364,19 @@ __device__ int match_event(const DevParams& P, const MatchIO& M, int VS, unsigne
                     }
                 }
             }
-        }
-        __syncthreads();
-        for (int s = tid; s < ns; s += T) {
-            if (M.velo_idx[row(s)] <= -2) {
-                M.velo_idx[row(s)] = -1;
-                M.chi2[row(s)] = 0.f;
+            __syncthreads();
+            for (int s = tid; s < ns; s += T) {
+                const int v = M.velo_idx[row(s)];
+                if (v <= -2) {
+                    M.velo_idx[row(s)] = -1;
+                    M.chi2[row(s)] = 0.f;
+                }
+                nl += v >= 0;
             }
         }
-        __syncthreads();
+    } else if (!plain) {
+        for (int s = tid; s < ns; s += T) nl += M.velo_idx[row(s)] >= 0;
     }
-    int nl = 0;
-    for (int s = tid; s < ns; s += T) nl += M.velo_idx[row(s)] >= 0;
     nl = warp_sum(nl);
     if ((tid & 31) == 0 && nl) atomicAdd(s_cnt, nl);
     __syncthreads();

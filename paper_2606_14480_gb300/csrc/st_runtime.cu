@@ -493,7 +493,7 @@ struct st_ctx {
     SeedShape big;                 // for the costliest items of a batch that may hold large events
     cudaStream_t side = nullptr;   // their launches run beside the others'
     cudaEvent_t ev_fork = nullptr, ev_started = nullptr, ev_join = nullptr;
-    int match_bps = 0;
+    int match_bps = 0, match_bps_large = 0;  // of the configured CTAs, and of the largest
     Pipeline* pipe = nullptr;
     std::mutex pipe_mu;
     bool timing = false;
@@ -718,6 +718,7 @@ extern "C" int st_create(const st_config* cfg, int device, st_ctx** out) {
     // and 893, 512 threads 814 and 946)
     if (c.threads_seed <= 256) ctx->big = seed_shape(1024, false, 8192, 1024, true);
     ctx->match_bps = match_blocks_per_sm(c.threads_match, ctx->match_smem, c.final_sel != 0);
+    ctx->match_bps_large = match_blocks_per_sm(kMaxThreads, ctx->match_smem, c.final_sel != 0);
     *out = ctx;
     return ST_OK;
 }
@@ -963,8 +964,16 @@ static int run_matching(st_ctx* ctx, Workspace& w, const st_velo& V, const st_se
     m.ghost_prob = L.ghost_prob;
     m.velo_smem = ctx->velo_smem;
     m.counters = ctx->counters;
-    int mbps = std::max(1, ctx->match_bps);
-    if (ctx->cfg.ctas_per_sm > 0) mbps = std::min(mbps, ctx->cfg.ctas_per_sm);
+    // Batches that the largest CTAs take in one round run in those (one event's
+    // latency falls with the threads that share it): 100 Run-3-like events 12.6
+    // us with 256 threads, 10.8 with 512, 300 uneven ones (120 tracks on average)
+    // 94 and 58 us; with more events than that the smaller ones' rounds win (600
+    // events 15 and 21 us).  A set ctas_per_sm asks for the configured CTAs.
+    int threads = ctx->cfg.threads_match, mbps = std::max(1, ctx->match_bps);
+    if (ctx->cfg.ctas_per_sm > 0)
+        mbps = std::min(mbps, ctx->cfg.ctas_per_sm);
+    else if (threads < kMaxThreads && V.n_events <= int64_t(ctx->n_sms) * ctx->match_bps_large)
+        threads = kMaxThreads, mbps = ctx->match_bps_large;
     const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(V.n_events, int64_t(ctx->n_sms) * mbps)));
     m.queue = nullptr;
     if (grid < V.n_events) {
@@ -972,7 +981,7 @@ static int run_matching(st_ctx* ctx, Workspace& w, const st_velo& V, const st_se
         ST_CUDA(ctx, cudaMemsetAsync(m.queue, 0, sizeof(int32_t), s));
     }
     tmark(ctx, w, 3, 0, s);
-    ST_CUDA(ctx, launch_match(ctx->P, m, grid, ctx->cfg.threads_match, s));
+    ST_CUDA(ctx, launch_match(ctx->P, m, grid, threads, s));
     tmark(ctx, w, 3, 1, s);
     return ST_OK;
 }

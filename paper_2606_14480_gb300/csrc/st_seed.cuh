@@ -24,10 +24,11 @@
 namespace st {
 
 // Registers per thread of each shape, for five, four, three and two CTAs per
-// SM.  Set outright: asked for as a number of CTAs per SM (launch bounds), the
-// same counts gave code that was slower everywhere (1000 Run-3-like events 232
-// against 215 us, 301 by direct calls 107 against 101, HLT2-style 250 events
-// 137 against 129).
+// SM.  Set outright next to the largest CTA: asked for as a number of CTAs per
+// SM, or without the largest CTA, the same counts give code that is slower
+// everywhere (1000 Run-3-like events 232 against 215 us, 301 by direct calls 107
+// against 101, HLT2-style 250 events 137 against 129).  (nvcc takes the pair
+// where both depend on a template's arguments.)
 constexpr int kSeedRegs256 = 48;
 constexpr int kSeedRegs256w = 64;
 constexpr int kSeedRegs384 = 56;

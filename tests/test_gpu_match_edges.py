@@ -1,5 +1,6 @@
-"""The UT search at the edges of its layout: hits around what shared memory
-holds and batches of several rounds."""
+"""Matching and UT search at the edges of their layouts: VELO segments in
+chunks of 512 and off 16-byte alignment, larger CTAs for small batches, UT hits
+around what shared memory holds and batches of several rounds."""
 
 import numpy as np
 import pytest
@@ -14,12 +15,53 @@ import oracle  # noqa: E402
 import parity  # noqa: E402
 from conftest import workload  # noqa: E402
 from paper_2606_14480_gb300 import st  # noqa: E402
-from synth import calibrate_zmatch  # noqa: E402
+from synth import calibrate_zmatch, ghost_nn_weights, make_events  # noqa: E402
 
 
 @pytest.fixture(scope="module")
 def zmx():
     return calibrate_zmatch(7826.0)
+
+
+@pytest.mark.parametrize("mode", [{}, dict(velo_unique=1), dict(final_sel=1)], ids=["plain", "unique", "final"])
+def test_match_layouts(mode, zmx):
+    """Chunk edges, an unaligned VELO array and other CTA shapes: the same pairs."""
+    counts = [0, 1, 64, 511, 512, 513, 1024, 1100]
+    b = make_events(len(counts), seed=4101, tracks=("fixed", 150))
+    rng = np.random.default_rng(4102)
+    velo = np.concatenate([b.velo[rng.integers(0, len(b.velo), n)] * np.float32(1 if n < 65 else 1.0001)
+                           for n in counts]).astype(np.float32)
+    for e, n in enumerate(counts):  # each event's own segments first
+        o, k = sum(counts[:e]), min(n, int(b.velo_off[e + 1] - b.velo_off[e]))
+        velo[o:o + k] = b.velo[b.velo_off[e]:b.velo_off[e] + k]
+    vo = np.concatenate([[0], np.cumsum(counts)])
+    db = st.DeviceBatch(b.ev_off, b.x, b.zone, vo, velo)
+    ref = None
+    for shape in ({}, dict(ctas_per_sm=1), dict(threads_match=64, ctas_per_sm=8), dict(threads_match=512)):
+        for shift in (0, 1):
+            flat = torch.zeros(4 * len(velo) + 1, device="cuda")
+            flat[shift:shift + 4 * len(velo)] = torch.as_tensor(velo.reshape(-1), device="cuda")
+            v = st.StVelo(len(counts), db.velo_s.ev_off, flat.data_ptr() + 4 * shift)
+            _, gcfg = parity.config_pair(zmx, **mode, **shape)
+            ctx = st.Context(gcfg)
+            if mode.get("final_sel"):
+                ctx.st_set_ghost_nn(ghost_nn_weights())
+            out = st.DeviceOutputs(len(counts), 8192)
+            ctx.seeding_run(db.hits, out.seeds)
+            ctx.matching_run(v, out.seeds, out.long)
+            r = out.to_numpy()
+            ctx.close()
+            n = int(r["ev_off"][-1])
+            for e in range(len(counts)):
+                idx = r["velo_idx"][r["ev_off"][e]:r["ev_off"][e + 1]]
+                assert r["n_long"][e] == (idx >= 0).sum() and (idx < counts[e]).all()
+            keys = ("velo_idx", "chi2") + (("ghost_prob",) if mode.get("final_sel") else ())
+            got = [r[k][:n] for k in keys] + [r["n_long"]]
+            if ref is None:
+                ref = got
+                assert r["n_long"][3:].min() > 0
+            for a, c in zip(ref, got):
+                assert np.array_equal(a, c), (shape, shift)
 
 
 @pytest.mark.parametrize("nu", [0, 1, 767, 768, 769, 4096, 4097])
