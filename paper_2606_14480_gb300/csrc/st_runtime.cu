@@ -1284,6 +1284,7 @@ struct OutBlock {
 struct Request {
     uint64_t id = 0;
     int64_t n_events = 0, n_hits = 0, n_velo = 0;
+    int64_t max_hits = 1;                  // of its events
     size_t h_off = 0, v_off = 0;           // offsets in the hit / VELO rings
     uint64_t h_id = 0, v_id = 0;           // ring blocks
     std::vector<int64_t> ev_off, velo_off;  // rebased to 0
@@ -1393,7 +1394,7 @@ static void slot_free(Slot& S) {
 static void launch_slot(st_ctx* ctx, Pipeline& pl, int si, std::unique_lock<std::mutex>& lk) {
     Slot& S = pl.slots[si];
     S.reqs.clear();
-    int64_t ne = 0, nh = 0, nv = 0;
+    int64_t ne = 0, nh = 0, nv = 0, max_hits = 1;
     size_t next_h = 0, next_v = 0;
     while (!pl.pending.empty()) {
         auto& r = pl.pending.front();
@@ -1408,6 +1409,7 @@ static void launch_slot(st_ctx* ctx, Pipeline& pl, int si, std::unique_lock<std:
         ne += r->n_events;
         nh += r->n_hits;
         nv += r->n_velo;
+        max_hits = std::max(max_hits, r->max_hits);
         next_h = r->h_off + size_t(r->n_hits);
         next_v = r->v_off + size_t(r->n_velo);
         S.reqs.push_back(r);
@@ -1451,11 +1453,14 @@ static void launch_slot(st_ctx* ctx, Pipeline& pl, int si, std::unique_lock<std:
     };
     ck(cudaMemcpyAsync(S.d_ev_off, S.h_ev_off, 8 * (ne + 1), cudaMemcpyHostToDevice, st));
     ck(cudaMemcpyAsync(S.d_velo_off, S.h_velo_off, 8 * (ne + 1), cudaMemcpyHostToDevice, st));
-    st_hits H{ne, S.d_ev_off, pl.d_x, pl.d_zone, nullptr, nullptr, pl.pc.max_hits_per_event, 0};
+    // the launch's own largest event and hit count: with the pipeline's limits
+    // instead, a container CTA took the shared memory of the largest event
+    // allowed (1500 Run-3-like events in six requests: 752 against 731 us)
+    st_hits H{ne, S.d_ev_off, pl.d_x, pl.d_zone, nullptr, nullptr, static_cast<int32_t>(max_hits), 0};
     st_seeds Sd{ob->cap, ob->ev_off, ob->hits, ob->params, ob->state, ob->n, ob->status};
     st_velo V{ne, S.d_velo_off, pl.d_velo};
     st_long L{ob->vidx, ob->chi2, ob->n_long, ob->gp};
-    if (rc == ST_OK) rc = run_batch(ctx, S.ws, H, Sd, V, L, st, pl.pc.max_hits_per_slot, false, false);
+    if (rc == ST_OK) rc = run_batch(ctx, S.ws, H, Sd, V, L, st, nh, false, false);
     ck(cudaMemcpyAsync(S.h_counts, ob->ev_off, 4 * (ne + 1), cudaMemcpyDeviceToHost, st));
     ck(cudaEventRecord(S.ev, st));
     S.rc = rc;
@@ -1642,6 +1647,7 @@ extern "C" int pipeline_submit(st_ctx* ctx, const st_hits* hh, const st_velo* hv
         if (dh < 0 || dv < 0) return set_err(ctx, ST_EINVAL, "pipeline_submit: decreasing offsets");
         if (dh > pl.pc.max_hits_per_event || dv > pl.pc.max_velo_per_event)
             return set_err(ctx, ST_OVERFLOW, "pipeline_submit: event larger than the pipeline limits");
+        r->max_hits = std::max(r->max_hits, dh);
     }
     if (n > pl.pc.max_events_per_slot || r->n_hits > pl.pc.max_hits_per_slot || r->n_velo > pl.pc.max_velo_per_slot)
         return set_err(ctx, ST_OVERFLOW, "pipeline_submit: batch larger than a pipeline slot");
