@@ -138,8 +138,10 @@ class ClockSampler:
 
 def kernel_source_hash():
     h = hashlib.sha256()
-    for f in ("st_kernels.cu", "st_device.cuh", "st_kernels.cuh"):
-        h.update(open(os.path.join(ROOT, "paper_2606_14480_gb300", "csrc", f), "rb").read())
+    d = os.path.join(ROOT, "paper_2606_14480_gb300", "csrc")
+    for f in sorted(os.listdir(d)):
+        if f.endswith(".cuh") or f.startswith(("st_seed", "st_kernels")):
+            h.update(open(os.path.join(d, f), "rb").read())
     return h.hexdigest()[:16]
 
 
@@ -323,11 +325,11 @@ def main():
     ctx.st_set_timing(False)
     graph = ctx.st_graph_create(db.hits, db.velo_s, out.seeds, out.long)
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)
-    # build, order, seed, scan, gather, and match unless the matching runs
-    # inside the seeding kernel (the HLT1 configuration with CTAs of at most
-    # 256 threads, without final selection or velo_unique)
-    fused = cfg.threads_seed <= 256 and cfg.iter_mode == 0 and not cfg.final_sel and not cfg.velo_unique
-    kernels_per_step = 5 if fused else 6
+    # build, order, seed, gather, a scan above 2048 events, and match unless the
+    # matching runs inside the seeding kernel (the HLT1 configuration without
+    # final selection)
+    fused = cfg.iter_mode == 0 and not cfg.final_sel
+    kernels_per_step = 4 + (n_ev > 2048) + (not fused)
 
     # ---------------- batched: graph replay, inputs resident in HBM
     with torch.cuda.stream(stream):
@@ -533,7 +535,7 @@ def main():
         pe_ms = marks[0].elapsed_time(marks[-1])
         per = np.array([a.elapsed_time(b) for a, b in zip(marks, marks[1:])])
         result["per_event"] = {"value": pe / (pe_ms / 1000.0), "unit": "events/s", "events_timed": pe,
-                               "launches_per_event": 6,
+                               "launches_per_event": 4,
                                "completion_gap_p50_ms": float(np.percentile(per, 50)),
                                "completion_gap_p99_ms": float(np.percentile(per, 99)),
                                "mode": "seeding_run + matching_run per event, one stream, back to back (the gap "

@@ -323,8 +323,10 @@ k_build(const __grid_constant__ DevParams P, const __grid_constant__ BuildArgs A
 // results are gathered per event.
 constexpr int kOrderThreads = 1024;
 // The items for the larger CTAs of a split batch: those that cost this many
-// times the mean.  2000 uneven events (120 tracks on average) / 500 of them, at
-// 4, 5, 6.5 times: 698 / 483, 679 / 492, 664 / 503 us.
+// times the mean (500 uneven events of 120 tracks on average at 4, 5, 6.5, 8
+// times: 483, 492, 503, 534 us) and at least as much as a CTA's share of the
+// batch; what costs less is done before the batch is in any CTA (10,000 uneven
+// events with 5, 8 times the mean alone 2918, 2801 us; 2733 unsplit).
 constexpr float kBigCost = 5.f;
 
 __global__ void __launch_bounds__(kOrderThreads) k_order(const __grid_constant__ BuildArgs A) {
@@ -365,7 +367,7 @@ __global__ void __launch_bounds__(kOrderThreads) k_order(const __grid_constant__
         for (int c = tid; c < kCostClasses; c += 32) sum += cost(c) * float(A.class_count[c]);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        const float bar = kBigCost * sum / float(items);
+        const float bar = fmaxf(kBigCost * sum / float(items), sum / float(A.n_ctas));
         int n = 0;
         for (int c = tid; c < kCostClasses; c += 32) n += cost(c) >= bar ? A.class_count[c] : 0;
         n = __reduce_add_sync(0xffffffffu, n);

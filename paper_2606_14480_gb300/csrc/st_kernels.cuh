@@ -37,7 +37,10 @@ struct BuildArgs {
     int32_t* class_count; // [128] items per class, zero before the launch
     int32_t* class_fill;  // [128] places taken per class, zero before the launch
     int32_t* order;       // [2 n_events] the seeding items, costliest class first; null: not needed
-    int32_t* n_big = nullptr;  // (k_order) out: the items at the front of `order` that cost kBigCost times the mean
+    // (k_order) out: the items at the front of `order` that cost kBigCost times the mean, and no less than the
+    // share of one of n_ctas CTAs
+    int32_t* n_big = nullptr;
+    int32_t n_ctas = 0;
     int32_t* queue;
     unsigned long long* counters;
 };

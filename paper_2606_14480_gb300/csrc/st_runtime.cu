@@ -577,7 +577,9 @@ static size_t carve(st_ctx* ctx, Workspace& w, int64_t ne, int64_t nh, int32_t m
         return base ? base + o : nullptr;
     };
     const int build_ctas = ctx->n_sms * kBuildCtasPerSm;
-    const int seed_ctas = ctx->n_sms * std::max(1, ctx->shape[0].bps);
+    // (split batches: one more for the larger CTA of each SM)
+    const int seed_ctas =
+        ctx->n_sms * (std::max(1, ctx->shape[0].bps) + (&w == &ctx->ws && mh > kBuildSmemHits && ctx->big.bps > 0));
     const int64_t items = 2 * ne;
     char* q = take(kQueueBytes + sizeof(int32_t) * size_t(items));  // zeroed per launch as one range
     char* cx = take(sizeof(float) * size_t(nh + 3 * ne + 8));
@@ -713,9 +715,9 @@ extern "C" int st_create(const st_config* cfg, int device, st_ctx** out) {
         return ST_ECUDA;
     }
     ctx->n_shapes = seed_shapes(c, ctx->shape, true);
-    // 48 registers a thread: a smaller CTA still fits beside it (with 64, alone
-    // on its SM, the split batches above take 746 and 896 us; 768 threads 758
-    // and 893, 512 threads 814 and 946)
+    // 48 registers a thread: a smaller CTA still fits beside it (2000 uneven
+    // events 679 us; with 64, alone on its SM, 746; 768 threads 758, 512 threads
+    // 814)
     if (c.threads_seed <= 256) ctx->big = seed_shape(1024, false, 8192, 1024, true);
     ctx->match_bps = match_blocks_per_sm(c.threads_match, ctx->match_smem, c.final_sel != 0);
     ctx->match_bps_large = match_blocks_per_sm(kMaxThreads, ctx->match_smem, c.final_sel != 0);
@@ -774,10 +776,11 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
     // batches are split: their large events and costliest items go to larger
     // CTAs (1024 threads, one per SM) in launches of their own on a side stream,
     // and the others follow once those CTAs have begun, so that every SM takes
-    // one of each.  2000 events of 120 tracks on average, up to 800: 1286 us in
-    // one launch, 679 us split; 400 events of 500 tracks 938 and 820 us.  The
-    // line is the size from which containers leave the smaller CTAs' shared
-    // memory.  Not on the serving pipeline's slots, whose streams run beside
+    // one of each.  Uneven events of 120 tracks on average, up to 800, in one
+    // launch and split: 500 events 1040 and 486 us, 2000 events 1410 and 632,
+    // 5000 events 1754 and 1406, 10,000 events 2740 and 2668; 400 events of 500
+    // tracks 886 and 830 us, 3000 of 400 tracks 2842 and 2857.  The line is the
+    // size from which containers leave the smaller CTAs' shared memory.  Not on the serving pipeline's slots, whose streams run beside
     // each other already, and not below one item per SM, where 512 threads serve
     // every item.
     const bool split = &w == &ctx->ws && 2 * H.n_events > ctx->n_sms && c.ctas_per_sm == 0 && ctx->big.bps > 0 &&
@@ -830,6 +833,7 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
     if (split) {
         b.split_hits = kBuildSplitHits;
         b.n_big = w.queues + 7;
+        b.n_ctas = g_seed;
         BuildArgs l = b;
         l.smem_hits = std::min<int>(H.max_hits_per_event, kBuildLargeHits);
         l.bins = std::min(bins_for(1, H.max_hits_per_event), kBuildLargeBins);
