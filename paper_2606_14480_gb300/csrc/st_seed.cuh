@@ -15,7 +15,8 @@
 // collect the rest before the expensive step, so that it runs with full warps.
 // 1000 Run-3-like events in one graph, matching fused in: the step 263 us when
 // every thread walked its own run of pairs and combinations to the end (k_seed
-// 206 us, 158 M warp instructions), 233 us this way (k_seed 190 us).
+// 206 us, 158 M warp instructions), 233 us this way (k_seed 190 us), 213 us with
+// the registers set as below (k_seed 171 us, 125 M warp instructions).
 #pragma once
 
 #include "st_common.cuh"
@@ -23,8 +24,8 @@
 
 namespace st {
 
-// Registers per thread of each shape, for five, four, three and two CTAs per
-// SM.  Set outright next to the largest CTA: asked for as a number of CTAs per
+// Registers per thread of each shape, for five, four, three, two and one CTAs
+// per SM.  Set outright next to the largest CTA: asked for as a number of CTAs per
 // SM, or without the largest CTA, the same counts give code that is slower
 // everywhere (1000 Run-3-like events 232 against 215 us, 301 by direct calls 107
 // against 101, HLT2-style 250 events 137 against 129).  (nvcc takes the pair
