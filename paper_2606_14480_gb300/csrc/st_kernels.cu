@@ -542,6 +542,7 @@ k_match(const __grid_constant__ DevParams P, const __grid_constant__ MatchArgs A
     __shared__ int s_item, s_cnt;
     ull ctr[4] = {0, 0, 0, 0};  // grid pairs, preselected pairs, Long tracks, evaluated pairs
     const MatchIO M{A.velo, A.seed_state, A.seed_n, A.velo_idx, A.chi2, A.ghost_prob};
+    pdl_wait();  // the seeds
 
     // the first event is the CTA's own number, the others come from the queue
     // (none without one: the grid covers the events)
@@ -669,12 +670,9 @@ cudaError_t launch_gather(const GatherArgs& a, cudaStream_t s, bool chained) {
     return launch_k(k, static_cast<unsigned>(grid), 256, 0, s, own ? chained : true, nullptr, a);
 }
 
-cudaError_t launch_match(const DevParams& P, const MatchArgs& a, int grid, int threads, cudaStream_t s) {
-    if (P.final_sel)
-        k_match<true><<<grid, threads, match_smem_bytes(a.velo_smem), s>>>(P, a);
-    else
-        k_match<false><<<grid, threads, match_smem_bytes(a.velo_smem), s>>>(P, a);
-    return cudaGetLastError();
+cudaError_t launch_match(const DevParams& P, const MatchArgs& a, int grid, int threads, cudaStream_t s, bool chained) {
+    return launch_k(P.final_sel ? k_match<true> : k_match<false>, static_cast<unsigned>(grid),
+                    static_cast<unsigned>(threads), match_smem_bytes(a.velo_smem), s, chained, nullptr, P, a);
 }
 
 }  // namespace st

@@ -170,7 +170,7 @@ cudaError_t launch_order(const BuildArgs& a, cudaStream_t s, bool chained = true
 cudaError_t launch_seed(const DevParams& P, const SeedArgs& a, int grid, int threads, bool wide, size_t smem,
                         cudaStream_t s, bool chained = true, cudaEvent_t started = nullptr);
 cudaError_t launch_gather(const GatherArgs& a, cudaStream_t s, bool chained = true);
-cudaError_t launch_match(const DevParams& P, const MatchArgs& a, int grid, int threads, cudaStream_t s);
+cudaError_t launch_match(const DevParams& P, const MatchArgs& a, int grid, int threads, cudaStream_t s, bool chained);
 
 // A launch as a programmatic dependent of the stream's previous kernel
 // (chained), or a plain one; `started` (if given) is recorded when all its
