@@ -121,7 +121,7 @@ k_build(const __grid_constant__ DevParams P, const __grid_constant__ BuildArgs A
     // the first warp: the next event and its offsets.  Tickets, or the next
     // large one of every gridDim.x-th event, 32 of them looked at together.
     __shared__ long long s_scan;
-    auto next_item = [&]() {
+    auto next_item = [&](bool first = false) {
         if constexpr (kLarge) {
             int64_t e = A.n_events;
             int64_t h0 = 0, h1 = 0;
@@ -151,12 +151,16 @@ k_build(const __grid_constant__ DevParams P, const __grid_constant__ BuildArgs A
             }
             __syncwarp();
         } else if (tid == 0) {
-            const int q = atomicAdd(A.queue, 1);
+            // its own number first, then tickets (one event by direct calls: 54
+            // us with a ticket each, 53 us without)
+            const int64_t q = first ? blockIdx.x
+                              : gridDim.x < A.n_events ? gridDim.x + int64_t(atomicAdd(A.queue, 1))
+                                                       : A.n_events;
             if (q < A.n_events) {
                 s_h0 = A.ev_off[q];
                 s_h1 = A.ev_off[q + 1];
             }
-            s_item = q;
+            s_item = static_cast<int>(q);
         }
     };
     if (tid == 0) {
@@ -165,7 +169,7 @@ k_build(const __grid_constant__ DevParams P, const __grid_constant__ BuildArgs A
     }
     if (tid < 32) {
         __syncwarp();
-        next_item();
+        next_item(true);
     }
 
     for (;;) {
