@@ -580,7 +580,14 @@ constexpr int kTripPerCand = 2;  // triplets of one round per candidate slot, ab
 // thread likewise.
 constexpr int kPairQueue = 64;
 constexpr int kTripQueue = 128;
-constexpr int kWalk = 12;
+constexpr int kWalk = 24;
+// Rounds with more pairs per first hit than kDensePairs, whose pairs find more
+// triplets each, walk fewer groups, so that the queues seldom run over.  1000
+// Run-3-like events (13 pairs per first hit): 220 us with 8 groups, 213 with 12,
+// 211 with 16, 210 with 24; 300 events by direct calls 98, 98, 96, 94 us; 2000
+// uneven events 642, 633, 650, 680 us, 627 with this rule.
+constexpr int kWalkDense = 12;
+constexpr int kDensePairs = 24;
 constexpr int kUvBlock = 1024;
 
 // Shared memory that the phases of an item use in turn: the warps' queues of
@@ -782,7 +789,7 @@ __device__ __forceinline__ bool xz_search(const DevParams& P, const SeedItem& it
         // groups of 32 pairs, none across two iterations
         const int G1 = (sg1 + 31) >> 5, G2 = G1 + ((sg2 - sg1 + 31) >> 5), G = G2 + ((tot_p - sg2 + 31) >> 5);
         int round_trips = 0;
-        int K = kWalk * n_warps;  // groups of a block walk
+        int K = (tot_p <= kDensePairs * n_own ? kWalk : kWalkDense) * n_warps;  // groups of a block walk
         int resume = 0;           // triplets already taken of a single group that has more than a queue holds
         for (int B = 0; B < G;) {
             const int nB = min(K, G - B);

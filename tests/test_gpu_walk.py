@@ -1,6 +1,6 @@
 """The block-wide walk of the seeding kernel at its edges.
 
-Pairs are walked in groups of 32 and blocks of 12 groups per warp, triplets
+Pairs are walked in groups of 32 and blocks of 12 or 24 groups per warp, triplets
 wait in queues of 128 per warp, UV combinations go in blocks of 1024, and
 batches of up to ten items per SM run in larger CTAs or with more registers.  Wide third-hit bands and
 windows, tiny events and batch sizes around that limit reach every branch; the
