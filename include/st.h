@@ -15,6 +15,8 @@
  *    during the call only, unless stated otherwise.
  *  - Work is enqueued on the caller's CUDA stream (cudaStream_t passed as
  *    void*; NULL = legacy default stream) and is asynchronous unless stated.
+ *    Batches that may hold large events use a stream of the context beside it,
+ *    which the caller's stream forks to and joins within the call.
  *  - Indices of hits are event-local: 0 .. hits-of-the-event-1, in the
  *    caller's order.  Seeds and VELO states are likewise event-local.
  *  - Per-event problems (invalid hit, capacity exceeded) are reported in the
