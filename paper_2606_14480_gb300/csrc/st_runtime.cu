@@ -501,15 +501,32 @@ struct st_ctx {
     int64_t wait_ns = kDefaultWaitNs;  // fused seeding kernel: longest wait for an announced event
     cudaEvent_t tev[4][2] = {};
     bool tused[4] = {};
+};
 
-    // the side stream takes up after what s holds now; s goes on after both
-    cudaError_t fork(cudaStream_t s) {
-        const cudaError_t e = cudaEventRecord(ev_fork, s);
-        return e != cudaSuccess ? e : cudaStreamWaitEvent(side, ev_fork, 0);
+// Work on the context's side stream beside stream s: it takes up after what s
+// holds at the fork, and s goes on after both from the join on, which is made
+// on every way out of the call: what a failed call had already given the side
+// stream still uses the workspace that the next call clears.
+struct Beside {
+    st_ctx* ctx;
+    cudaStream_t s;
+    bool open = false;
+
+    Beside(st_ctx* c, cudaStream_t st) : ctx(c), s(st) {}
+    Beside(const Beside&) = delete;
+    ~Beside() {
+        if (open) join();
     }
-    cudaError_t join(cudaStream_t s) {
-        const cudaError_t e = cudaEventRecord(ev_join, side);
-        return e != cudaSuccess ? e : cudaStreamWaitEvent(s, ev_join, 0);
+    cudaError_t fork() {
+        cudaError_t e = cudaEventRecord(ctx->ev_fork, s);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
+        open = e == cudaSuccess;
+        return e;
+    }
+    cudaError_t join() {
+        open = false;
+        const cudaError_t e = cudaEventRecord(ctx->ev_join, ctx->side);
+        return e != cudaSuccess ? e : cudaStreamWaitEvent(s, ctx->ev_join, 0);
     }
 };
 
@@ -829,6 +846,7 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
     // at saturation).
     const bool marks = ctx->timing && &w == &ctx->ws;
     const bool chain = &w == &ctx->ws;
+    Beside beside(ctx, s);
     tmark(ctx, w, 0, 0, s);
     if (split) {
         b.split_hits = kBuildSplitHits;
@@ -837,13 +855,13 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
         BuildArgs l = b;
         l.smem_hits = std::min<int>(H.max_hits_per_event, kBuildLargeHits);
         l.bins = std::min(bins_for(1, H.max_hits_per_event), kBuildLargeBins);
-        ST_CUDA(ctx, ctx->fork(s));
+        ST_CUDA(ctx, beside.fork());
         ST_CUDA(ctx, launch_build_large(ctx->P, l, static_cast<int>(std::min<int64_t>(H.n_events, ctx->n_sms)),
                                         ctx->side, ctx->ev_started));
         ST_CUDA(ctx, cudaStreamWaitEvent(s, ctx->ev_started, 0));
     }
     ST_CUDA(ctx, launch_build(ctx->P, b, g_build, c.threads_build, s));
-    if (split) ST_CUDA(ctx, ctx->join(s));
+    if (split) ST_CUDA(ctx, beside.join());
     ST_CUDA(ctx, launch_order(b, s, chain && !split));
     tmark(ctx, w, 0, 1, s);
 
@@ -907,7 +925,7 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
         l.part = 1;
         l.n_big = b.n_big;
         l.queue = w.queues + 10;
-        ST_CUDA(ctx, ctx->fork(s));
+        ST_CUDA(ctx, beside.fork());
         ST_CUDA(ctx, launch_seed(ctx->P, l, g_big, big.threads, big.wide, big.smem, ctx->side, false, ctx->ev_started));
         ST_CUDA(ctx, cudaStreamWaitEvent(s, ctx->ev_started, 0));
         a.part = 2;
@@ -916,7 +934,7 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
         g_seed = std::min(g_seed, w.seed_ctas - g_big);
     }
     ST_CUDA(ctx, launch_seed(ctx->P, a, g_seed, sh.threads, sh.wide, sh.smem, s, chain && !marks && !split));
-    if (split) ST_CUDA(ctx, ctx->join(s));
+    if (split) ST_CUDA(ctx, beside.join());
     tmark(ctx, w, 1, 1, s);
 
     GatherArgs g;
