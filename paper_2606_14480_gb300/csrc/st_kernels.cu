@@ -650,8 +650,9 @@ cudaError_t launch_order(const BuildArgs& a, cudaStream_t s, bool chained) {
 cudaError_t launch_seed(const DevParams& P, const SeedArgs& a, int grid, int threads, bool wide, size_t smem,
                         cudaStream_t s, bool chained, cudaEvent_t started) {
     const bool sq = P.iter_mode == 1;
-    if (a.velo && sq) return cudaErrorInvalidValue;  // the runtime asks for fused matching in the HLT1 mode only
-    const SeedKernel k = seed_kernel(threads, wide, sq, a.velo != nullptr);
+    const bool fused = a.ev_done != nullptr;  // (a batch without any VELO segment may have no array of them)
+    if (fused && sq) return cudaErrorInvalidValue;  // the runtime asks for fused matching in the HLT1 mode only
+    const SeedKernel k = seed_kernel(threads, wide, sq, fused);
     return launch_k(k, static_cast<unsigned>(grid), static_cast<unsigned>(threads), smem, s, chained, started, P, a);
 }
 

@@ -81,7 +81,7 @@ struct SeedArgs {
     int32_t* retry_ctr = nullptr;
     int32_t* queue;
     unsigned long long* counters;
-    // matching fused into the seeding kernel (velo null: seeding only): the
+    // matching fused into the seeding kernel (ev_done null: seeding only): the
     // CTA that finishes an event's second half matches the event, or near
     // the end announces it for CTAs without seeding work
     const int64_t* velo_off = nullptr;

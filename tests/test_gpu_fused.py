@@ -143,3 +143,24 @@ def test_fused_full_size_uneven_equals_two_step(zmx):
     assert (got["status"] == 0).all()
     for k in ref:
         assert np.array_equal(ref[k], got[k]), k
+
+
+@pytest.mark.parametrize("threads", [256, 512])
+def test_no_velo_array(threads, zmx):
+    """A graph of events without VELO segments, whose array of them is null:
+    no seed has a Long track."""
+    b = workload("run3", n_events=40)
+    _, gcfg = parity.config_pair(zmx, threads_seed=threads)
+    ctx = st.Context(gcfg)
+    db = st.DeviceBatch(b.ev_off, b.x, b.zone, np.zeros(41, np.int64), np.zeros((0, 4), np.float32))
+    out = st.DeviceOutputs(40, max(1024, b.n_hits // 4))
+    for a in (out.velo_idx, out.chi2, out.n_long):
+        a.fill_(7)
+    g = ctx.st_graph_create(db.hits, st.StVelo(40, db.velo_off.data_ptr(), None), out.seeds, out.long)
+    g.st_graph_launch()
+    torch.cuda.synchronize()
+    r = out.to_numpy()
+    g.close()
+    ctx.close()
+    assert r["ev_off"][-1] > 1000 and (r["status"] == 0).all()
+    assert (r["velo_idx"] == -1).all() and (r["chi2"] == 0).all() and (r["n_long"] == 0).all()
