@@ -585,8 +585,10 @@ static int bins_for(int64_t n_events, int64_t n_hits) {
     return b;
 }
 
-// Arena layout for the given capacities; assigns pointers if `base`.
-static size_t carve(st_ctx* ctx, Workspace& w, int64_t ne, int64_t nh, int32_t mh, int64_t sc, char* base) {
+// Arena layout for the given capacities, with `large` also one seeding slot per
+// SM for the larger CTAs of split batches; assigns pointers if `base`.
+static size_t carve(st_ctx* ctx, Workspace& w, int64_t ne, int64_t nh, int32_t mh, int64_t sc, bool large,
+                    char* base) {
     size_t off = 0;
     auto take = [&](size_t bytes) {
         size_t o = off;
@@ -594,9 +596,7 @@ static size_t carve(st_ctx* ctx, Workspace& w, int64_t ne, int64_t nh, int32_t m
         return base ? base + o : nullptr;
     };
     const int build_ctas = ctx->n_sms * kBuildCtasPerSm;
-    // (split batches: one more for the larger CTA of each SM)
-    const int seed_ctas =
-        ctx->n_sms * (std::max(1, ctx->shape[0].bps) + (&w == &ctx->ws && mh > kBuildSmemHits && ctx->big.bps > 0));
+    const int seed_ctas = ctx->n_sms * (std::max(1, ctx->shape[0].bps) + large);
     const int64_t items = 2 * ne;
     char* q = take(kQueueBytes + sizeof(int32_t) * size_t(items));  // zeroed per launch as one range
     char* cx = take(sizeof(float) * size_t(nh + 3 * ne + 8));
@@ -657,7 +657,8 @@ static int ensure(st_ctx* ctx, Workspace& w, int64_t ne, int64_t nh, int32_t mh,
     nh = std::max(nh, w.cap_hits);
     mh = std::max(mh, w.cap_max_hits);
     sc = std::max(sc, w.cap_seeds);
-    const size_t need = carve(ctx, w, ne, nh, mh, sc, nullptr);
+    bool large = &w == &ctx->ws && mh > kBuildSmemHits && ctx->big.bps > 0;
+    size_t need = carve(ctx, w, ne, nh, mh, sc, large, nullptr);
     if (w.base) {
         cudaError_t e = cudaDeviceSynchronize();
         if (e != cudaSuccess) return set_err(ctx, ST_ECUDA, "cudaDeviceSynchronize: %s", cudaGetErrorString(e));
@@ -666,10 +667,17 @@ static int ensure(st_ctx* ctx, Workspace& w, int64_t ne, int64_t nh, int32_t mh,
     }
     char* p = nullptr;
     cudaError_t e = cudaMalloc(&p, need);
+    if (e == cudaErrorMemoryAllocation && large) {
+        // the larger CTAs can also have slots of the others
+        cudaGetLastError();
+        large = false;
+        need = carve(ctx, w, ne, nh, mh, sc, large, nullptr);
+        e = cudaMalloc(&p, need);
+    }
     if (e != cudaSuccess) return set_err(ctx, ST_ENOMEM, "cudaMalloc(%zu): %s", need, cudaGetErrorString(e));
     w.base = p;
     w.bytes = need;
-    carve(ctx, w, ne, nh, mh, sc, p);
+    carve(ctx, w, ne, nh, mh, sc, large, p);
     return ST_OK;
 }
 
@@ -1595,7 +1603,7 @@ static int pipeline_configure_locked(st_ctx* ctx, const st_pipeline_config* pcin
     Workspace t;
     const int64_t ocap = out_cap_for(pc.max_hits_per_slot);
     const size_t ws_bytes = carve(ctx, t, pc.max_events_per_slot, pc.max_hits_per_slot, pc.max_hits_per_event,
-                                  ocap, nullptr);
+                                  ocap, false, nullptr);
     const size_t in_bytes = 2 * (8 * size_t(pc.max_hits_per_slot) + 16 * size_t(pc.max_velo_per_slot));
     const size_t out_bytes = 2 * out_block_bytes(pc.max_events_per_slot, ocap);
     const size_t per_slot = ws_bytes + in_bytes + out_bytes;

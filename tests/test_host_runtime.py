@@ -1,6 +1,6 @@
 """The host runtime (st_runtime.cu) without a GPU, linked with a stand-in for
 the CUDA runtime and the kernel launchers (fake_cuda.cpp, fake_launch.cu): what a call leaves
-behind when a launch in its middle fails."""
+behind when a launch in its middle fails, and what scratch it makes do with."""
 
 import ctypes as C
 import os
@@ -79,4 +79,28 @@ def test_split_batch_joins_after_a_failed_launch(rt):
         assert rt.fake_unjoined(s) == 0, chain[k]
     rt.fake_reset(-1, -1)
     assert ctx.seeding_run(500, 16384, s) == st.ST_OK and names(rt) == chain
+    ctx.close()
+
+
+def test_split_batch_without_room_for_its_own_slots(rt):
+    """Where device memory has no room for the scratch of the larger CTAs, a
+    batch with large events runs as split with what the ordinary CTAs have."""
+    used = []
+    for max_hits in (6144, 6145):
+        ctx = Ctx(rt)
+        before = rt.fake_used()
+        assert ctx.seeding_run(500, max_hits, None) == st.ST_OK
+        used.append(rt.fake_used() - before)
+        chain = names(rt)
+        ctx.close()
+    assert used[1] - used[0] > 50 << 20 and "seed_large" in chain
+    ctx = Ctx(rt)
+    rt.fake_reset(-1, rt.fake_used() + used[1] - (50 << 20))
+    assert ctx.seeding_run(500, 6145, None) == st.ST_OK and names(rt) == chain
+    rt.fake_reset(-1, rt.fake_used())  # (nothing more is allocated)
+    assert ctx.seeding_run(500, 6145, None) == st.ST_OK
+    ctx.close()
+    ctx = Ctx(rt)
+    rt.fake_reset(-1, rt.fake_used() + used[0] // 2)
+    assert ctx.seeding_run(500, 6145, None) == st.ST_ENOMEM
     ctx.close()
