@@ -765,7 +765,8 @@ __device__ __forceinline__ bool xz_search(const DevParams& P, const SeedItem& it
             const int st3 = szl[I.s3], n3 = szl[I.s3 + 1] - st3;
             const HitMap m3 = map.zone(I.s3);
             const int lo3 = zlo(X + st3, m3, n3, xc - I.dx3);
-            np = zhi(X + st3, m3, n3, xc + I.dx3) - lo3;
+            // (a window may end before it starts: layers against the flight direction, a negative scale)
+            np = max(zhi(X + st3, m3, n3, xc + I.dx3) - lo3, 0);
             if (is_used(used, szl[I.s1] + k1)) np = 0;
             p3 = st3 + lo3;
             own1 = k1;

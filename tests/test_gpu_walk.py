@@ -59,6 +59,25 @@ def test_walk_edges_parity_and_shapes(n, tracks, over, zmx):
             assert np.array_equal(other[k], gpu[k]), (shape, k)
 
 
+@pytest.mark.parametrize("over", [
+    dict(iter_layers=[[0, 4, 11], [11, 7, 3], [0, 7, 11]]),  # the second iteration's windows are empty
+    dict(iter_layers=[[11, 7, 3], [0, 4, 11], [0, 7, 11]]),  # the first one's
+    dict(iter_layers=[[0, 4, 11], [11, 7, 3], [0, 7, 11]], n_iter=3),
+    dict(dx3_scale=-1.0),                                     # all of them
+])
+def test_empty_two_hit_windows(over, zmx):
+    """Two-hit windows that end before they start hold no hit and take nothing
+    from the other iterations'."""
+    b = make_events(6, seed=4031, tracks=("fixed", 60))
+    ocfg, gcfg = parity.config_pair(zmx, **over)
+    gpu, cnt = run_gpu(b, gcfg)
+    assert (gpu["status"] == 0).all()
+    rep = parity.compare_seeding(gpu, ocfg, b)
+    assert rep.agreement >= parity.AGREE_MIN and not rep.untraced and not rep.bad_params, rep.summary()
+    none = "dx3_scale" in over
+    assert (gpu["ev_off"][-1] == 0) == none and (cnt["pairs"] == 0) == none
+
+
 @pytest.mark.parametrize("items", [2, 3, 4, 10])
 @pytest.mark.parametrize("mode", [{}, dict(uv_mode=1), dict(iter_mode=1)], ids=["hlt1", "hough", "seq"])
 def test_larger_ctas_give_the_same(mode, items, zmx):
