@@ -538,8 +538,10 @@ __global__ void __launch_bounds__(256, 8) k_gather(const __grid_constant__ Gathe
 // per-event CSR layout.
 // kFinal: compiled with the final selection of Section 4.4 (the plain
 // instantiation does not carry its registers).
-template <bool kFinal>
-__global__ void __launch_bounds__(kMaxThreads)
+// kMany: CTAs of up to 256 threads with 40 registers each, six to an SM, where
+// the 51 registers otherwise taken leave room for four.
+template <bool kFinal, bool kMany>
+__global__ void __launch_bounds__(kMany ? kMatchManyThreads : kMaxThreads, kMany ? 6 : 0)
 k_match(const __grid_constant__ DevParams P, const __grid_constant__ MatchArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int tid = threadIdx.x;
@@ -578,14 +580,19 @@ size_t match_smem_bytes(int velo_smem) { return match_smem_size(velo_smem); }
 // launchers
 // ===========================================================================
 
+typedef void (*MatchKernel)(const DevParams, const MatchArgs);
+static MatchKernel match_kernel(bool final_sel, bool many) {
+    return final_sel ? k_match<true, false> : many ? k_match<false, true> : k_match<false, false>;
+}
+
 // Raise each kernel's dynamic shared-memory ceiling to what the device allows
 // next to the kernel's own static shared memory (opt-in maximum - static).
 cudaError_t set_smem_limits(size_t optin) {
-    const void* fns[4 + 3 * kSeedShapes] = {reinterpret_cast<const void*>(k_build<false>),
-                                            reinterpret_cast<const void*>(k_build<true>),
-                                            reinterpret_cast<const void*>(k_match<false>),
-                                            reinterpret_cast<const void*>(k_match<true>)};
-    int n = 4;
+    const void* fns[5 + 3 * kSeedShapes] = {
+        reinterpret_cast<const void*>(k_build<false>), reinterpret_cast<const void*>(k_build<true>),
+        reinterpret_cast<const void*>(match_kernel(false, false)), reinterpret_cast<const void*>(match_kernel(true, false)),
+        reinterpret_cast<const void*>(match_kernel(false, true))};
+    int n = 5;
     for (int sh = 0; sh < kSeedShapes; ++sh)
         for (int mode = 0; mode < 3; ++mode)
             fns[n++] = reinterpret_cast<const void*>(seed_kernel(kSeedThreads[sh], kSeedWide[sh], mode == 1, mode == 2));
@@ -621,12 +628,9 @@ int seed_blocks_per_sm(int threads, bool wide, size_t smem) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, seed_kernel(threads, wide, false, false), threads, smem);
     return n;
 }
-int match_blocks_per_sm(int threads, size_t smem, bool final_sel) {
+int match_blocks_per_sm(int threads, size_t smem, bool final_sel, bool many) {
     int n = 0;
-    if (final_sel)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_match<true>, threads, smem);
-    else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_match<false>, threads, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, match_kernel(final_sel, many), threads, smem);
     return n;
 }
 
@@ -675,9 +679,10 @@ cudaError_t launch_gather(const GatherArgs& a, cudaStream_t s, bool chained) {
     return launch_k(k, static_cast<unsigned>(grid), 256, 0, s, own ? chained : true, nullptr, a);
 }
 
-cudaError_t launch_match(const DevParams& P, const MatchArgs& a, int grid, int threads, cudaStream_t s, bool chained) {
-    return launch_k(P.final_sel ? k_match<true> : k_match<false>, static_cast<unsigned>(grid),
-                    static_cast<unsigned>(threads), match_smem_bytes(a.velo_smem), s, chained, nullptr, P, a);
+cudaError_t launch_match(const DevParams& P, const MatchArgs& a, int grid, int threads, bool many, cudaStream_t s,
+                         bool chained) {
+    return launch_k(match_kernel(P.final_sel != 0, many), static_cast<unsigned>(grid), static_cast<unsigned>(threads),
+                    match_smem_bytes(a.velo_smem), s, chained, nullptr, P, a);
 }
 
 }  // namespace st

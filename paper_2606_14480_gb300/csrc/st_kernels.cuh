@@ -170,7 +170,8 @@ cudaError_t launch_order(const BuildArgs& a, cudaStream_t s, bool chained = true
 cudaError_t launch_seed(const DevParams& P, const SeedArgs& a, int grid, int threads, bool wide, size_t smem,
                         cudaStream_t s, bool chained = true, cudaEvent_t started = nullptr);
 cudaError_t launch_gather(const GatherArgs& a, cudaStream_t s, bool chained = true);
-cudaError_t launch_match(const DevParams& P, const MatchArgs& a, int grid, int threads, cudaStream_t s, bool chained);
+cudaError_t launch_match(const DevParams& P, const MatchArgs& a, int grid, int threads, bool many, cudaStream_t s,
+                         bool chained);
 
 // A launch as a programmatic dependent of the stream's previous kernel
 // (chained), or a plain one; `started` (if given) is recorded when all its
@@ -200,7 +201,8 @@ static cudaError_t launch_k(void (*k)(KArgs...), unsigned grid, unsigned threads
 // occupancy helpers
 int build_blocks_per_sm(int threads, size_t smem);
 int seed_blocks_per_sm(int threads, bool wide, size_t smem);
-int match_blocks_per_sm(int threads, size_t smem, bool final_sel);
+constexpr int kMatchManyThreads = 256;  // most threads of a k_match CTA of which many fit on an SM
+int match_blocks_per_sm(int threads, size_t smem, bool final_sel, bool many);
 cudaError_t set_smem_limits(size_t optin);
 cudaError_t smem_limits_hold(size_t optin, bool& hold);
 

@@ -494,6 +494,7 @@ struct st_ctx {
     cudaStream_t side = nullptr;   // their launches run beside the others'
     cudaEvent_t ev_fork = nullptr, ev_started = nullptr, ev_join = nullptr;
     int match_bps = 0, match_bps_large = 0;  // of the configured CTAs, and of the largest
+    int match_bps_many = 0;                  // of the configured CTAs with fewer registers (0: there are none)
     Pipeline* pipe = nullptr;
     std::mutex pipe_mu;
     bool timing = false;
@@ -744,8 +745,10 @@ extern "C" int st_create(const st_config* cfg, int device, st_ctx** out) {
     // events 679 us; with 64, alone on its SM, 746; 768 threads 758, 512 threads
     // 814)
     if (c.threads_seed <= 256) ctx->big = seed_shape(1024, false, 8192, 1024, true);
-    ctx->match_bps = match_blocks_per_sm(c.threads_match, ctx->match_smem, c.final_sel != 0);
-    ctx->match_bps_large = match_blocks_per_sm(kMaxThreads, ctx->match_smem, c.final_sel != 0);
+    ctx->match_bps = match_blocks_per_sm(c.threads_match, ctx->match_smem, c.final_sel != 0, false);
+    ctx->match_bps_large = match_blocks_per_sm(kMaxThreads, ctx->match_smem, c.final_sel != 0, false);
+    if (c.threads_match <= kMatchManyThreads && !c.final_sel)
+        ctx->match_bps_many = match_blocks_per_sm(c.threads_match, ctx->match_smem, false, true);
     *out = ctx;
     return ST_OK;
 }
@@ -1002,12 +1005,25 @@ static int run_matching(st_ctx* ctx, Workspace& w, const st_velo& V, const st_se
     // latency falls with the threads that share it): 100 Run-3-like events 12.6
     // us with 256 threads, 10.8 with 512, 300 uneven ones (120 tracks on average)
     // 94 and 58 us; with more events than that the smaller ones' rounds win (600
-    // events 15 and 21 us).  A set ctas_per_sm asks for the configured CTAs.
+    // events 15 and 21 us).  Batches that need two rounds of these and one of the
+    // same CTAs with fewer registers (six to an SM against four) run in the
+    // latter, and so do batches of more than two and a half rounds of those, which
+    // the throughput decides: 620 Run-3-like events 15.6 us against 20.7, 900 events
+    // 18.0 / 22.9, 2400 40.9 / 43.3, 8000 107 / 117; 900 uneven events, which wait
+    // for their largest, 98.9 / 97.6.  In between the events' evenness decides
+    // (1300 events 26.9 / 29.0, uneven ones 111.7 / 110.0; 2000 events 37.2 / 37.4,
+    // uneven ones 115.8 / 113.2).  A set ctas_per_sm asks for the configured CTAs.
     int threads = ctx->cfg.threads_match, mbps = std::max(1, ctx->match_bps);
-    if (ctx->cfg.ctas_per_sm > 0)
+    bool many = false;
+    const int64_t round = int64_t(ctx->n_sms) * mbps, round_many = int64_t(ctx->n_sms) * ctx->match_bps_many;
+    if (ctx->cfg.ctas_per_sm > 0) {
         mbps = std::min(mbps, ctx->cfg.ctas_per_sm);
-    else if (threads < kMaxThreads && V.n_events <= int64_t(ctx->n_sms) * ctx->match_bps_large)
+    } else if (threads < kMaxThreads && V.n_events <= int64_t(ctx->n_sms) * ctx->match_bps_large) {
         threads = kMaxThreads, mbps = ctx->match_bps_large;
+    } else if (round_many > round && V.n_events > round &&
+               (V.n_events <= round_many || 2 * V.n_events > 5 * round_many)) {
+        many = true, mbps = ctx->match_bps_many;
+    }
     const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(V.n_events, int64_t(ctx->n_sms) * mbps)));
     m.queue = nullptr;
     if (grid < V.n_events) {
@@ -1016,7 +1032,7 @@ static int run_matching(st_ctx* ctx, Workspace& w, const st_velo& V, const st_se
     }
     const bool marks = ctx->timing && &w == &ctx->ws;
     tmark(ctx, w, 3, 0, s);
-    ST_CUDA(ctx, launch_match(ctx->P, m, grid, threads, s, chained && !m.queue && !marks));
+    ST_CUDA(ctx, launch_match(ctx->P, m, grid, threads, many, s, chained && !m.queue && !marks));
     tmark(ctx, w, 3, 1, s);
     return ST_OK;
 }

@@ -16,7 +16,7 @@ int build_blocks_per_sm(int, size_t) { return 4; }
 int seed_blocks_per_sm(int threads, bool wide, size_t) {
     return threads <= 256 ? (wide ? 4 : 5) : threads <= 384 ? 3 : threads <= 512 ? 2 : 1;
 }
-int match_blocks_per_sm(int threads, size_t, bool) { return threads <= 256 ? 5 : 2; }
+int match_blocks_per_sm(int threads, size_t, bool, bool many) { return threads > 256 ? 2 : many ? 6 : 4; }
 cudaError_t set_smem_limits(size_t) { return cudaSuccess; }
 cudaError_t launch_build(const DevParams&, const BuildArgs&, int, int, cudaStream_t s) { return fake_launch("build", s, nullptr); }
 cudaError_t launch_build_large(const DevParams&, const BuildArgs&, int, cudaStream_t s, cudaEvent_t started) {
@@ -28,6 +28,8 @@ cudaError_t launch_seed(const DevParams&, const SeedArgs& a, int, int, bool, siz
     return fake_launch(a.part == 1 ? "seed_large" : "seed", s, started);
 }
 cudaError_t launch_gather(const GatherArgs&, cudaStream_t s, bool) { return fake_launch("gather", s, nullptr); }
-cudaError_t launch_match(const DevParams&, const MatchArgs&, int, int, cudaStream_t s, bool) { return fake_launch("match", s, nullptr); }
+cudaError_t launch_match(const DevParams&, const MatchArgs&, int, int, bool many, cudaStream_t s, bool) {
+    return fake_launch(many ? "match_many" : "match", s, nullptr);
+}
 cudaError_t launch_ut(const UtParams&, const UtArgs&, int, cudaStream_t s, bool) { return fake_launch("ut", s, nullptr); }
 }  // namespace st

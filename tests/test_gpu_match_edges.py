@@ -64,6 +64,26 @@ def test_match_layouts(mode, zmx):
                 assert np.array_equal(a, c), (shape, shift)
 
 
+@pytest.mark.parametrize("per_sm", [4, 6, 15])
+@pytest.mark.parametrize("mode", [{}, dict(velo_unique=1)], ids=["plain", "unique"])
+def test_match_rounds(mode, per_sm, zmx):
+    """On both sides of the batch sizes at which the matching takes CTAs with
+    fewer registers: the pairs are those of the configured CTAs."""
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+    b = make_events(n + 1, seed=4104, tracks=("fixed", 12))
+    for k in (n, n + 1):
+        db = st.DeviceBatch.from_synth(b.subset(range(k)))
+        res = []
+        for shape in (dict(ctas_per_sm=8), {}):
+            _, gcfg = parity.config_pair(zmx, **mode, **shape)
+            ctx = st.Context(gcfg)
+            res.append(st.run_batch(ctx, db).to_numpy())
+            ctx.close()
+        assert res[0]["n_long"].sum() > k
+        for key in ("velo_idx", "chi2", "n_long"):
+            assert np.array_equal(res[0][key], res[1][key]), (k, key)
+
+
 @pytest.mark.parametrize("nu", [0, 1, 767, 768, 769, 4096, 4097])
 def test_ut_sizes(nu, zmx):
     """UT hits of an event around the threads' shares and shared memory."""
