@@ -585,7 +585,12 @@ constexpr int kWalk = 24;
 // triplets each, walk fewer groups, so that the queues seldom run over.  1000
 // Run-3-like events (13 pairs per first hit): 220 us with 8 groups, 213 with 12,
 // 211 with 16, 210 with 24; 300 events by direct calls 98, 98, 96, 94 us; 2000
-// uneven events 642, 633, 650, 680 us, 627 with this rule.
+// uneven events 642, 633, 650, 680 us, 627 with this rule.  Where a queue runs
+// over all the same (wide bands), the walk is repeated with as many groups as the
+// triplets found say, and the item's next walks follow their own counts: a
+// quarter of the groups for the rest of a round, as before, made 300 events with
+// the band up to 20 times the expected curvature 210 us, 167 this way, 5 times
+// 133 and 121.
 constexpr int kWalkDense = 12;
 constexpr int kDensePairs = 24;
 constexpr int kUvBlock = 1024;
@@ -662,7 +667,7 @@ struct SeedVars {
     int item, match, cnt;
     int nvalid, nlist;
     int seg[2];        // first pair or combination of a round's second and third part
-    int wcnt[32];      // triplets queued per warp
+    int wcnt[32];      // triplets found per warp
 };
 
 // What the phases of an item share.
@@ -741,6 +746,7 @@ __device__ __forceinline__ bool xz_search(const DevParams& P, const SeedItem& it
     uint2* const tqs = reinterpret_cast<uint2*>(M.phase);  // the warps' queues: triplets, then pairs
     uint2* const tq = tqs + kTripQueue * wid;
     uint32_t* const pq = reinterpret_cast<uint32_t*>(tqs + kTripQueue * n_warps) + kPairQueue * wid;
+    int K = kWalk * n_warps;  // groups of a block's next walk
     int n_items = 0;
     for (int it = it_lo; it < it_hi; ++it) n_items += szl[P.it[it].s1 + 1] - szl[P.it[it].s1];
     for (int b1 = 0; b1 < n_items; b1 += R) {
@@ -790,13 +796,14 @@ __device__ __forceinline__ bool xz_search(const DevParams& P, const SeedItem& it
         // groups of 32 pairs, none across two iterations
         const int G1 = (sg1 + 31) >> 5, G2 = G1 + ((sg2 - sg1 + 31) >> 5), G = G2 + ((tot_p - sg2 + 31) >> 5);
         int round_trips = 0;
-        int K = (tot_p <= kDensePairs * n_own ? kWalk : kWalkDense) * n_warps;  // groups of a block walk
+        const int most = (tot_p <= kDensePairs * n_own ? kWalk : kWalkDense) * n_warps;
+        K = min(K, most);
         int resume = 0;           // triplets already taken of a single group that has more than a queue holds
         for (int B = 0; B < G;) {
             const int nB = min(K, G - B);
             const int per = (nB + n_warps - 1) / n_warps;
             const int gb = B + min(per * wid, nB), ge = B + min(per * (wid + 1), nB);
-            int tn = 0, all = 0;  // triplets queued; found
+            int all = 0;  // triplets found
 #pragma unroll 1
             for (int it = it_lo; it < it_hi; ++it) {
                 const int gs = it == it_lo ? 0 : it == it_lo + 1 ? G1 : G2, gt = it == it_lo ? G1 : it == it_lo + 1 ? G2 : G;
@@ -870,15 +877,21 @@ __device__ __forceinline__ bool xz_search(const DevParams& P, const SeedItem& it
                     __syncwarp();
                 }
             }
-            tn = min(max(all - resume, 0), kTripQueue);
-            if (lane == 0) V.wcnt[wid] = tn;
-            const bool more = __syncthreads_or(all - resume > kTripQueue);
-            if (more && nB > 1) {  // some warp's queue was too short: fewer groups at a time
-                K = max(1, nB / 4);
-                continue;
+            if (lane == 0) V.wcnt[wid] = max(all - resume, 0);
+            const bool more = __syncthreads_or(all - resume > kTripQueue);  // some warp's queue was too short
+            int wb = lane < n_warps ? V.wcnt[lane] : 0;
+            if (more || K < most) {
+                // the next walk takes as many groups as fill three quarters of
+                // the queue of the warp with most triplets
+                const int fit = per * (kTripQueue * 3 / 4) / max(__reduce_max_sync(0xffffffffu, wb), 1);
+                K = more && per == 1 ? max(1, nB / 4) : min(max(fit, 1) * n_warps, most);
+                if (more && nB > 1) {
+                    __syncthreads();  // (the counts' last reads)
+                    continue;
+                }
+                wb = min(wb, kTripQueue);
             }
             // the queued triplets, one to a thread
-            int wb = lane < n_warps ? V.wcnt[lane] : 0;
             const int nt = __reduce_add_sync(0xffffffffu, wb);
 #pragma unroll
             for (int s = 1; s < 32; s <<= 1) {
