@@ -7,6 +7,7 @@ paper_2606_14480_gb300/libst.so (CUDA runtime linked statically).
 from __future__ import annotations
 
 import os
+import re
 import shutil
 import subprocess
 import sys
@@ -35,6 +36,21 @@ def _deps():
     return max(os.path.getmtime(f) for f in files)
 
 
+def check_seed_registers(log: str) -> int:
+    """Checks `ptxas -v` output: every k_seed<threads, registers, ..> in it
+    keeps to its registers, on which the CTAs per SM and with them the launch
+    shapes rest.  Returns how many it saw."""
+    seen = 0
+    for name, used in re.findall(r"Compiling entry function '(\S+)'.*?Used (\d+) registers", log, re.S):
+        m = re.search(r"k_seedILi(\d+)ELi(\d+)E", name)
+        if m:
+            seen += 1
+            if int(used) > int(m.group(2)):
+                raise RuntimeError(f"k_seed for {m.group(1)} threads takes {used} registers a thread, "
+                                   f"not {m.group(2)}: {name}")
+    return seen
+
+
 def build(force: bool = False, verbose: bool = False, extra=()) -> str:
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _deps():
         return LIB
@@ -44,12 +60,15 @@ def build(force: bool = False, verbose: bool = False, extra=()) -> str:
 
     def compile_one(src):
         obj = os.path.join(BUILD, src.replace(".cu", ".o"))
-        cmd = common + ["-c", os.path.join(CSRC, src), "-o", obj]
+        seed = re.fullmatch(r"st_seed\d+w?\.cu", src)
+        cmd = common + (["-Xptxas", "-v"] if seed else []) + ["-c", os.path.join(CSRC, src), "-o", obj]
         if verbose:
             print(" ".join(cmd), file=sys.stderr)
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed for {src}:\n{r.stdout}\n{r.stderr}")
+        if seed and not check_seed_registers(r.stdout + r.stderr):
+            raise RuntimeError(f"no register counts of k_seed in the compiler's output for {src}")
         return obj
 
     with ThreadPoolExecutor(len(SOURCES)) as ex:

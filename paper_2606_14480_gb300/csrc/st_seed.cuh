@@ -29,7 +29,8 @@ namespace st {
 // SM, or without the largest CTA, the same counts give code that is slower
 // everywhere (1000 Run-3-like events 232 against 215 us, 301 by direct calls 107
 // against 101, HLT2-style 250 events 137 against 129).  (nvcc takes the pair
-// where both depend on a template's arguments.)
+// where both depend on a template's arguments; the two are not documented to go
+// together, so the build checks the registers that come out.)
 constexpr int kSeedRegs256 = 48;
 constexpr int kSeedRegs256w = 64;
 constexpr int kSeedRegs384 = 56;
@@ -1132,7 +1133,7 @@ __device__ __forceinline__ void uv_search(const DevParams& P, const SeedItem& it
 // GPU with others (the serving pipeline) do not defer: a waiting CTA would
 // hold resources the other kernels could use.
 template <int kT, int kR, bool kSeq, bool kFuse>
-__global__ void __launch_bounds__(kT) __maxnreg__(kR)
+__global__ void __launch_bounds__(kT) __maxnreg__(kR) 
 k_seed(const __grid_constant__ DevParams P, const __grid_constant__ SeedArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ SeedVars V;

@@ -102,3 +102,23 @@ int main(void) {
             C.sizeof(st.StLong), C.sizeof(st.StCounters), C.sizeof(st.StPipelineConfig),
             C.sizeof(st.StRequestInfo), st.StConfig.threads_seed.offset, st.StConfig.velo_unique.offset]
     assert got == want
+
+
+def test_build_checks_the_seeding_kernels_registers():
+    """The launch shapes rest on k_seed's registers per thread: the build takes
+    compiler output that keeps to them and refuses any other."""
+    from paper_2606_14480_gb300 import build
+    line = ("ptxas info    : Compiling entry function '{}' for 'sm_103a'\n"
+            "ptxas info    : Function properties for {}\n"
+            "    8 bytes stack frame, 12 bytes spill stores, 12 bytes spill loads\n"
+            "ptxas info    : Used {} registers, used 1 barriers\n")
+    seed = "_ZN2st6k_seedILi{}ELi{}ELb0ELb1EEEvNS_9DevParamsENS_8SeedArgsE"
+
+    def log(*kernels):
+        return "".join(line.format(n, n, r) for n, r in kernels)
+    other = ("_ZN2st7k_matchILb0ELb0EEEvNS_9DevParamsENS_9MatchArgsE", 200)
+    assert build.check_seed_registers(log(other)) == 0
+    assert build.check_seed_registers(log((seed.format(256, 48), 48), other, (seed.format(1024, 48), 40))) == 2
+    for t, r in ((256, 48), (256, 64), (1024, 48)):
+        with pytest.raises(RuntimeError, match=f"{t} threads"):
+            build.check_seed_registers(log(other, (seed.format(t, r), r + 8)))
