@@ -1133,7 +1133,7 @@ __device__ __forceinline__ void uv_search(const DevParams& P, const SeedItem& it
 // GPU with others (the serving pipeline) do not defer: a waiting CTA would
 // hold resources the other kernels could use.
 template <int kT, int kR, bool kSeq, bool kFuse>
-__global__ void __launch_bounds__(kT) __maxnreg__(kR) 
+__global__ void __launch_bounds__(kT) __maxnreg__(kR)
 k_seed(const __grid_constant__ DevParams P, const __grid_constant__ SeedArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ SeedVars V;

@@ -99,6 +99,28 @@ def test_tuned_windows_record():
     assert all(p["ms"] >= rec["ms"] for p in rec["grid"] if p["ok"])
 
 
+class _FakeBench:
+    """Times that drift: the first run is slow, later ones 2% faster, and only
+    smem_hits = 2048 is faster in earnest."""
+
+    def __init__(self):
+        self.n = 0
+
+    def run(self, cfg, keep_outputs):
+        self.n += 1
+        ms = (1.0 if self.n == 1 else 0.98) * (0.9 if cfg.smem_hits == 2048 else 1.0)
+        return ms, {"ev_off": np.zeros(1)} if keep_outputs else None
+
+
+def test_launch_tuning_does_not_pick_noise():
+    """Points that run the same launches as the start are not picked for a
+    faster timing of theirs; one that is faster each time is."""
+    space = {"threads_seed": (128, 256, 512), "threads_match": (128, 256, 512), "smem_hits": (1536, 2048)}
+    r = autotune.tune_launch({}, None, space=space, bench=_FakeBench())
+    assert r.best == {"threads_seed": 256, "threads_match": 256, "smem_hits": 2048}
+    assert all(p.ok for p in r.points)
+
+
 # ------------------------------------------------------------------- GPU
 
 def _gpu():
