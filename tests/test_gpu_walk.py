@@ -1,9 +1,10 @@
 """The block-wide walk of the seeding kernel at its edges.
 
 Pairs are walked in groups of 32 and blocks of 12 or 24 groups per warp, triplets
-wait in queues of 128 per warp, UV combinations go in blocks of 1024, and
-batches of up to ten items per SM run in larger CTAs or with more registers.  Wide third-hit bands and
-windows, tiny events and batch sizes around that limit reach every branch; the
+wait in queues of 128 per warp, UV combinations go in blocks of 1024.  Batches
+of up to four items per SM run in larger CTAs or with more registers, and so do
+those of more than five and up to eight, in two rounds.  Wide third-hit bands and
+windows, tiny events and batch sizes around these limits reach every branch; the
 oracle, and the same batch in CTAs of other sizes, say what is right."""
 
 import numpy as np
@@ -78,11 +79,11 @@ def test_empty_two_hit_windows(over, zmx):
     assert (gpu["ev_off"][-1] == 0) == none and (cnt["pairs"] == 0) == none
 
 
-@pytest.mark.parametrize("items", [2, 3, 4, 10])
+@pytest.mark.parametrize("items", [2, 3, 4, 5, 8])
 @pytest.mark.parametrize("mode", [{}, dict(uv_mode=1), dict(iter_mode=1)], ids=["hlt1", "hough", "seq"])
 def test_larger_ctas_give_the_same(mode, items, zmx):
-    """Around the largest batch (items per SM) that each kind of larger CTAs
-    takes: every event's result is that of the batch one event larger."""
+    """Around the batch sizes (items per SM) at which another kind of CTAs
+    begins: every event's result is that of the batch one event larger."""
     sms = items * torch.cuda.get_device_properties(0).multi_processor_count // 2
     b = workload("run3", n_events=sms + 1)
     big = run(b, zmx, **mode)
@@ -92,6 +93,32 @@ def test_larger_ctas_give_the_same(mode, items, zmx):
     for k in KEYS[1:]:
         assert np.array_equal(small[k], big[k][:len(small[k])]), k
     assert n > 0
+
+
+@pytest.mark.parametrize("mode", [{}, dict(uv_mode=1), dict(iter_mode=1)], ids=["hlt1", "hough", "seq"])
+def test_two_rounds_of_wider_ctas(mode, zmx):
+    """Between five and eight items per SM: the CTAs with more registers take
+    the items from the queue in cost order, and in a graph leave the last
+    events' matching to each other.  The results are those of the configured
+    CTAs (a set ctas_per_sm)."""
+    n = 13 * torch.cuda.get_device_properties(0).multi_processor_count // 4
+    b = workload("run3", n_events=n)
+    want = run(b, zmx, ctas_per_sm=5, **mode)
+    got = run(b, zmx, **mode)
+    _, gcfg = parity.config_pair(zmx, **mode)
+    ctx = st.Context(gcfg)
+    db = st.DeviceBatch.from_synth(b)
+    out = st.DeviceOutputs(n, max(1024, b.n_hits // 4))
+    gr = ctx.st_graph_create(db.hits, db.velo_s, out.seeds, out.long)
+    gr.st_graph_launch()
+    gr.st_graph_launch()
+    torch.cuda.synchronize()
+    graph = out.to_numpy()
+    gr.close()
+    ctx.close()
+    assert (want["status"] == 0).all() and want["ev_off"][-1] > 100 * n
+    for k in KEYS:
+        assert np.array_equal(want[k], got[k]) and np.array_equal(want[k], graph[k]), k
 
 
 def _concat(parts):
@@ -155,12 +182,45 @@ def test_large_events_beside_ordinary(mode, zmx):
                 assert np.array_equal(r[k], res[0][k]), (mh, k)
 
 
+def test_large_events_in_a_callers_capture(zmx):
+    """A batch that may hold large events, captured by the caller: the work on
+    the context's own stream becomes part of the caller's graph."""
+    s = make_events(200, seed=4024, tracks=("fixed", 30))
+    d = make_events(2, seed=4025, tracks=("fixed", 500))
+    eo, x, zone, vo, velo = _concat([(s, None), (d, None)])
+    n = len(eo) - 1
+    _, gcfg = parity.config_pair(zmx)
+    db = st.DeviceBatch(eo, x, zone, vo, velo)
+    assert db.max_hits > 6144
+    cap = 80 * n
+    ctx = st.Context(gcfg)
+    want = st.run_batch(ctx, db, cap=cap).to_numpy()
+    out = st.DeviceOutputs(n, cap)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        ctx.seeding_run(db.hits, out.seeds)
+        ctx.matching_run(db.velo_s, out.seeds, out.long)
+    for _ in range(2):
+        for a in (out.hits, out.velo_idx, out.n_long):
+            a.fill_(-7)
+        g.replay()
+        torch.cuda.synchronize()
+        got = out.to_numpy()
+        for k in KEYS:
+            assert np.array_equal(got[k], want[k]), k
+    del g
+    again = st.run_batch(ctx, db, cap=cap).to_numpy()
+    assert np.array_equal(again["hits"], want["hits"]) and want["ev_off"][-1] > 1000
+    ctx.close()
+
+
 @pytest.mark.parametrize("n,tracks,over", [
     (60, 150, {}),                                       # one CTA per item
     (20, 260, {}),                                       # halves with more hits than shared memory holds
     (48, 60, dict(m_lo=0.0, m_hi=40.0, chi2x_max=1e9)),  # more candidates than the first step's scratch holds
     (48, 60, dict(uv_tol=40.0, n_uv_min=2)),             # more UV combinations than it holds
     (48, 60, dict(iter_mode=1, uv_tol=40.0, n_uv_min=2)),
+    (48, 60, dict(uv_mode=1, uv_tol=10.0)),              # Hough hypotheses: more valid ones than it holds
 ])
 def test_static_entry_in_two_steps(n, tracks, over, zmx):
     """seeding_run_static runs the items with little scratch each first and
