@@ -97,7 +97,8 @@ typedef struct {
     int32_t threads_seed;      /* threads per CTA of the seeding kernel: 64, 128, 256, 512 (batches that
                                 * leave SMs idle take larger CTAs unless ctas_per_sm is set) */
     int32_t threads_build;     /* threads per CTA of the container kernel */
-    int32_t threads_match;     /* threads per CTA of the matching kernel */
+    int32_t threads_match;     /* threads per CTA of the matching kernel (batches that 512-thread CTAs take
+                                * in one round run in those unless ctas_per_sm is set) */
     int32_t ctas_per_sm;       /* persistent CTAs per SM (0 = occupancy maximum) */
     int32_t smem_hits;         /* hits of one detector half staged in shared memory */
     int32_t cand_cap;          /* x-z candidates per (event, half) work item */
@@ -136,7 +137,9 @@ typedef struct {
  * ev_off[0] need not be 0.  z and dxdy may be NULL; when given, each hit's
  * value must equal the configured value of its layer within 1e-3 mm / 1e-6,
  * else the event's status is ST_EINVAL.  max_hits_per_event is a host-side
- * bound; larger events get ST_OVERFLOW.  Events with a zone outside [0, 24)
+ * bound; larger events get ST_OVERFLOW.  It also sizes the launches: above
+ * 6144 the batch runs as one that may hold large events, which costs ordinary
+ * events 10 to 20 us more, so pass the largest event's size where it is known.  Events with a zone outside [0, 24)
  * or a non-finite x get ST_EINVAL. */
 typedef struct {
     int64_t n_events;
@@ -156,6 +159,8 @@ typedef struct {
  *   state   [cap*4]      float: x, y, tx, ty at z_state
  *   n_hits  [cap*2]      int8 : x-layer hits, stereo hits
  *   status  [n_events]   int32: ST_OK, ST_EINVAL or ST_OVERFLOW
+ * The halves of an event are searched apart: an event with ST_OVERFLOW may
+ * carry the seeds (and the Long tracks) of the half that did not overflow.
  * Within an event, seeds of half 0 precede those of half 1, each in the
  * deterministic order of the search (iteration, T1 hit, T3 hit, T2 hit). */
 typedef struct {
@@ -224,7 +229,9 @@ const char* st_last_error(const st_ctx* ctx);
 /* Pre-allocate scratch for batches of up to n_events events, n_hits hits,
  * max_hits_per_event hits per event and seeds_cap seeds, so that later
  * seeding_run / matching_run calls allocate nothing (required before CUDA
- * graph capture).  Synchronous. */
+ * graph capture).  With max_hits_per_event above 6144 the scratch holds one
+ * more seeding slot per SM (120 MB in all at the default cand_cap), or none
+ * more where the device has no room for them.  Synchronous. */
 int st_reserve(st_ctx* ctx, int64_t n_events, int64_t n_hits, int32_t max_hits_per_event,
                int64_t seeds_cap);
 
@@ -314,9 +321,10 @@ int st_set_ghost_nn(st_ctx* ctx, const float* weights, int32_t n);
  * first (st_reserve).  The arguments' pointers must stay valid while the
  * graph exists.  *out receives the graph; launch with st_graph_launch.
  * With iter_mode 0 and no final selection the matching runs inside the
- * seeding kernel (each event as soon as its two halves are seeded); the outputs are those of the two calls.  If that kernel ever gave
- * up a (bounded) wait for an event being seeded, which a correct run cannot
- * do, every event of the launch gets status ST_TIMEOUT.  The serving pipeline
+ * seeding kernel (each event as soon as its two halves are seeded); the
+ * outputs are those of the two calls.  If that kernel ever gave up a (bounded)
+ * wait for an event being seeded, which a correct run cannot do, every event
+ * of the launch gets status ST_TIMEOUT.  The serving pipeline
  * runs batches the same way. */
 int st_graph_create(st_ctx* ctx, const st_hits* hits, const st_velo* velo, st_seeds* seeds,
                     st_long* out, st_graph** graph);

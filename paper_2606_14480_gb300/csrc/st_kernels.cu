@@ -1,22 +1,26 @@
 // st_kernels.cu -- sm_103a kernels of the SciFi Seeding + VELO-SciFi Matching
-// hot path.  All kernels are persistent: a grid of (SMs x resident CTAs) pulls
-// work items (events, or detector halves of events) from a device counter.
+// hot path.  A batch that fits the resident CTAs gives each the work item
+// (event, or detector half) of its own number; for larger ones persistent CTAs
+// pull items from a device counter.
 //
 //   k_build   one event per item: validate hits, sort them by (container
 //             slot, x, index) with a bucketed rank sort in shared memory, write
 //             the per-event container (x, original index) and slot offsets.
-//   k_order   one CTA: the seeding items sorted by cost class, costliest
-//             first, the order in which k_seed's queue hands them out.
+//   k_order   the seeding items sorted by cost class, costliest first, the
+//             order in which k_seed's queue hands them out; left out where
+//             every item has a CTA of its own.
 //   k_seed    (st_seed.cuh) one detector half of one event per item (the
 //             paper keeps the halves apart, Section 5.2).  In the batch path
 //             the CTA that finishes an event's second half also matches the
 //             event.
-//   k_scan / k_gather   per-event CSR of the seed records.
-//   k_match   one event per item: VELO segments bucketed by ty in shared
-//             memory, one thread per seed for its lowest chi2_match, then
-//             optionally the final selection (ghost network, clones).
+//   k_scan / k_gather   per-event CSR of the seed records (up to 2048 events
+//             k_gather finds the events' places itself).
+//   k_match   (st_match.cuh) one event per item: VELO segments bucketed by ty
+//             in shared memory, up to eight lanes per seed for its lowest
+//             chi2_match, then optionally the final selection (ghost network,
+//             clones).
 //
-// k_order, k_seed, k_scan and k_gather are launched as programmatic
+// k_order, k_seed, k_scan, k_gather and k_match are launched as programmatic
 // dependents of the kernel before them in the stream: their CTAs may be
 // scheduled while it finishes, and wait (griddepcontrol.wait) for its
 // completion and its memory before they read or write anything it touches.

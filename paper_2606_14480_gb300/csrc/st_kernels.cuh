@@ -158,11 +158,11 @@ size_t seed_smem_limit_bytes(int threads, int smem_hits, int tbl_smem, int key_s
 size_t seed_slot_limit_bytes(int cand_cap, int max_xhits);
 size_t match_smem_bytes(int velo_smem);
 
-// chained: k_order, k_seed and k_scan are launched as programmatic dependents
-// of the stream's previous kernel (the caller puts no other stream work
-// between them; k_gather always follows k_scan that way).  Their CTAs may
-// then wait on the SMs for that kernel, which only pays where no other
-// stream's kernels want those SMs.
+// chained: k_order, k_seed, k_scan and k_gather are launched as programmatic
+// dependents of the stream's previous kernel (the caller puts no other stream
+// work between them; behind k_scan k_gather always is one), k_match of whatever
+// the stream holds.  Their CTAs may then wait on the SMs for that kernel, which
+// only pays where no other stream's kernels want those SMs.
 // started (may be null): recorded when all CTAs of the launch have begun.
 cudaError_t launch_build(const DevParams& P, const BuildArgs& a, int grid, int threads, cudaStream_t s);
 cudaError_t launch_build_large(const DevParams& P, const BuildArgs& a, int grid, cudaStream_t s, cudaEvent_t started);

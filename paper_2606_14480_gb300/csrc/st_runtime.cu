@@ -415,15 +415,14 @@ int seed_shapes(const st_config& c, SeedShape out[kSeedShapes], bool bps) {
 // the latency of one item, which falls with the threads that share it; above
 // that the SMs are shared anyway and the smaller CTAs pass their barriers
 // sooner.  Of the CTAs of 256 threads, four to an SM with 64 registers a thread
-// spill less (570 bytes against 840) than five with 48, which pays for up to two
-// rounds where they are as many as five to an SM need.  k_seed, Run-3-like events, at
-// 256 / 448 / 512 threads: 67 events 69 / 57 / 53 us, 150 events 90 / 71 / 65,
-// 220 events 91 / 81 / 85.  The whole step at 448 / 384 threads: 200 events 98 /
-// 95 us, 225 events 96 / 94; at 256 threads five / four to an SM: 250 events
-// 106 / 104, 300 events 112 / 109, 350 events 114 / 118, 450 events 131 / 130,
-// 600 events 151 / 146, 760 events 176 / 182, 900 events 202 / 202, 1000 events
-// 215 / 224, 2000 events 403 / 421.  A set ctas_per_sm asks for the configured
-// shape.
+// spill less than five with 48, which pays for up to two rounds where they are
+// as many as five to an SM need.  The whole step of Run-3-like events by a graph
+// at 256 threads five / four to an SM, 384 and 512 threads (us): 67 events 72 /
+// 70 / 65 / 62, 152 events 81 / 78 / 78 / 71, 228 events 94 / 91 / 88 / 101, 304
+// events 108 / 107 / 110 / 108, 350 events 106 / 114 / 118 / 129, 450 events 125 /
+// 124 / 125 / 144, 600 events 144 / 139 / 161 / 185, 760 events 169 / 175 / 198 /
+// 228, 1000 events 208 / 218 / 247 / 295, 2000 events 391 / 409 / 466 / 564.  A
+// set ctas_per_sm asks for the configured shape.
 const SeedShape& pick_seed_shape(const SeedShape* shapes, int n, const st_config& c, int64_t items, int n_sms,
                                  int64_t max_ctas) {
     auto ctas = [&](int k) { return std::min<int64_t>(int64_t(n_sms) * shapes[k].bps, max_ctas); };
@@ -797,7 +796,6 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
     const int sbps = c.ctas_per_sm > 0 ? std::min(std::max(1, sh.bps), c.ctas_per_sm) : std::max(1, sh.bps);
     int g_seed = static_cast<int>(std::max<int64_t>(
         1, std::min<int64_t>({2 * H.n_events, int64_t(ctx->n_sms) * sbps, int64_t(w.seed_ctas)})));
-    // every item has a CTA of its own from the start: no queue, no order
     // A batch that may hold events many times the ordinary size waits for its
     // largest items: one of 800 tracks took 1.1 ms in a CTA of 256 threads,
     // 630 us in one of 512, and its container 82 us in scratch memory.  Such
@@ -808,11 +806,16 @@ static int run_seeding(st_ctx* ctx, Workspace& w, const st_hits& H, st_seeds& S,
     // launch and split: 500 events 1040 and 486 us, 2000 events 1410 and 632,
     // 5000 events 1754 and 1406, 10,000 events 2740 and 2668; 400 events of 500
     // tracks 886 and 830 us, 3000 of 400 tracks 2842 and 2857.  The line is the
-    // size from which containers leave the smaller CTAs' shared memory.  Not on the serving pipeline's slots, whose streams run beside
-    // each other already, and not below one item per SM, where 512 threads serve
-    // every item.
+    // size from which containers leave the smaller CTAs' shared memory, and the
+    // caller's bound stands for the events, whose sizes only the device knows: with
+    // a bound above it ordinary events are split too (Run-3-like events by direct
+    // calls, with their own bound and one of 16384: 80 events 64 and 84 us, 300
+    // events 100 and 121, 1000 events 214 and 232).  Not on the serving pipeline's
+    // slots, whose streams run beside each other already, and not below one item
+    // per SM, where 512 threads serve every item.
     const bool split = &w == &ctx->ws && 2 * H.n_events > ctx->n_sms && c.ctas_per_sm == 0 && ctx->big.bps > 0 &&
                        H.max_hits_per_event > kBuildSmemHits && w.seed_ctas >= 3 * ctx->n_sms;
+    // every item has a CTA of its own from the start: no queue, no order
     const bool one_round = 2 * H.n_events <= g_seed && !split;
     const int build_cap = std::min<int>(H.max_hits_per_event, split ? kBuildSplitHits : kBuildSmemHits);
     const int bins = split ? bins_for(1, build_cap) : bins_for(H.n_events, n_hits_total);

@@ -12,8 +12,13 @@ size_t seed_slot_bytes(int cand_cap, int uv_cap, int tbl_cap, int max_hits) {
 }
 
 // The shared memory and the scratch per CTA that a configuration is accepted
-// by (no less than what the kernel takes of either): what the interface's
-// limits are stated in.
+// by: what an earlier layout of the kernel took (9216 bytes of bucket tables, 12
+// triplet keys per thread of 512, 40 bytes per stored UV combination, and so
+// on), in which the interface states its limits, so that what is accepted and
+// what is refused does not change with the layout.  The present one takes less
+// of both wherever a limit is near, but can take more of a small configuration
+// (512 threads without staged hits: 36 KB against 18): the callers take the
+// larger of this and what is really needed.
 size_t seed_smem_limit_bytes(int threads, int smem_hits, int tbl_smem, int key_smem) {
     return align16(sizeof(float) * smem_hits) + 9216 + sizeof(ull) * (tbl_smem + key_smem) +
            sizeof(float) * 6 * key_smem + sizeof(int) * 3 * threads + sizeof(int) * (36 + 16);

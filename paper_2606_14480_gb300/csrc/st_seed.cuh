@@ -356,7 +356,7 @@ __device__ __forceinline__ UV uv_unpack(const uint4 v) {
 // occupancy mask; a cluster b is bins (b, b+1), its population the number of
 // layers with a hit in it, counted for all clusters at once with three bit
 // planes.  The kept clusters (most populated first, at least n_uv_min, ties to
-// // the smaller b) go to hcl[8 j ..], their number to hn[j].  Six lanes per seed,
+// the smaller b) go to hcl[8 j ..], their number to hn[j].  Six lanes per seed,
 // one stereo layer each, whose masks they exchange; five seeds per warp.
 __device__ __forceinline__ void hough_select_in(const DevParams& P, const float* X, const int* szl, const HitMap map,
                                                 const uint32_t* used, const float* Xs, int h, int kb, int nk,
