@@ -79,11 +79,12 @@ def test_empty_two_hit_windows(over, zmx):
     assert (gpu["ev_off"][-1] == 0) == none and (cnt["pairs"] == 0) == none
 
 
-@pytest.mark.parametrize("items", [2, 3, 4, 5, 8])
+@pytest.mark.parametrize("items", [2, 3, 4, 5, 8, 10])
 @pytest.mark.parametrize("mode", [{}, dict(uv_mode=1), dict(iter_mode=1)], ids=["hlt1", "hough", "seq"])
 def test_larger_ctas_give_the_same(mode, items, zmx):
     """Around the batch sizes (items per SM) at which another kind of CTAs
-    begins: every event's result is that of the batch one event larger."""
+    begins, and one that the configured CTAs take either way: every event's
+    result is that of the batch one event larger."""
     sms = items * torch.cuda.get_device_properties(0).multi_processor_count // 2
     b = workload("run3", n_events=sms + 1)
     big = run(b, zmx, **mode)
